@@ -52,8 +52,8 @@ typedef enum {
   DICH_ERR_ARG = 1,           /* bad size, NULL / host / misaligned pointer, bad option */
   DICH_ERR_NOT_DOMINANT = 2,  /* |t_0| < |t_-1| + |t_1|: eq. 32-33 fails (not supported) */
   DICH_ERR_SINGULAR = 3,      /* t_0 = 0 with dominance, or a zero block pivot (Theorem 1) */
-  DICH_ERR_TIMEOUT = 4,       /* a bounded wait for a kernel's own bulk copies ran out (not
-                                 expected; no kernel waits on another CTA or rank) */
+  DICH_ERR_TIMEOUT = 4,       /* a device wait ran out (not expected: no kernel of this build waits
+                                 on anything but its own barriers) */
   DICH_ERR_NONFINITE = 5,     /* a NaN/Inf was produced on the device */
   DICH_ERR_CUDA = 6,          /* a CUDA runtime call failed; see dichotomy_last_cuda_error */
   DICH_ERR_ALIAS = 7,         /* output aliases an input */
@@ -86,9 +86,8 @@ enum {
                                         general matrices: any rows, judged by dich_plan_info.growth;
                                         check results with dichotomy_residual / dichotomy_gen_residual */
   /* MIXED-form window kernel of Toeplitz plans and batches (the results agree to rounding):
-   * the register path keeps a thread's two 16-row blocks in registers (bulk copies in and out,
-   * four CTAs per SM); the shared-memory path sweeps the window's tile in shared memory (six CTAs
-   * per SM).  Default: the register path for single plans, and for batches unless most of their
+   * the register path keeps a thread's two 16-row blocks in registers; the shared-memory path sweeps the window's tile in shared memory.
+   * Default: the register path for single plans, and for batches unless most of their
    * MIXED windows are whole one-window systems (latency-bound windows, where occupancy wins). */
   DICH_FLAG_REG_PATH = 32,           /* the register path wherever its window shape allows */
   DICH_FLAG_SMEM_PATH = 64           /* the shared-memory path for every window */

@@ -760,7 +760,7 @@ int dichotomy_plan_bind(dich_plan_t p, void* d_ws, size_t bytes, void* stream) {
 }
 
 // device_mem: F and x are device memory (false: mapped host memory, read and written by the kernels
-// over the host link), which lets aligned windows use bulk copies
+// over the host link), which may take the register path
 static int plan_launch(dich_plan_t p, const double* F, double* x, const double* xf, double* gt, bool adjoint,
                        cudaStream_t st, int64_t M = 1, int64_t ldf = 0, int64_t ldx = 0, int64_t win0 = 0,
                        int64_t nwin = -1, bool device_mem = true) {
@@ -791,9 +791,9 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   a.sys_offset = sys_offset;
   a.ldf = ldf;
   a.ldx = ldx;
-  // the register path (bulk copies) only for full solves of device memory, unless the plan asks
+  // the register path only for full solves of device memory, unless the plan asks
   // for the shared-memory path (the general path's passes always take that one)
-  a.bulk = (device_mem && p->path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? 1 : 0;
+  a.reg_path = (device_mem && p->path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? 1 : 0;
   const size_t smem = smem_bytes(p->NT, p->n_smem, p->form);
   // windows [win0, win0 + grid) of the single and halo paths (all of them unless a range is given)
   const int grid = (int)((nwin < 0) ? p->tiles : nwin);
@@ -1634,7 +1634,7 @@ static int batch_launch(dich_batch_t b, const double* F, double* x, const double
     a.check_finite = (b->opts.flags & DICH_FLAG_CHECK_FINITE) ? 1 : 0;
     a.n_smem = b->n_smem[f];
     a.sys_offset = sys_offset;
-    a.bulk = b->reg_path ? 1 : 0;   // batch vectors are device memory
+    a.reg_path = b->reg_path ? 1 : 0;   // batch vectors are device memory
     const size_t smem = smem_bytes(b->NT[f], a.n_smem, f);
     cudaError_t e = (f == FORM_F64) ? launch_window_f64(b->NT[f], (int)nitems, smem, sf, a)
                                     : launch_window_mixed(b->NT[f], (int)nitems, smem, sf, a);

@@ -60,7 +60,7 @@ enum Mode : int32_t {
 enum StatusBits : uint32_t {
   ST_NONFINITE = 1u,
   ST_SCHEDULE = 2u,
-  ST_TIMEOUT = 4u,    // a bounded wait for the CTA's own bulk copies ran out (the CTA stored nothing)
+  ST_TIMEOUT = 4u,    // a bounded wait ran out (no kernel of this build waits on anything but barriers)
 };
 
 // Device-side plan record of one system (256 bytes, 8-byte fields first).

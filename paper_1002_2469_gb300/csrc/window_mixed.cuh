@@ -370,11 +370,8 @@ __global__ void __launch_bounds__(NT, (KIND == KIND_REGADJ ? 512 : 768) / NT)
   const int len = nwin * n - (has_last ? (n - nlast) : 0);
 
   if constexpr (KIND == KIND_REG || KIND == KIND_REGADJ) {
-    // 16-row blocks, all of full size, 16-byte aligned device memory: the register path
-    if (A.bulk && A.mode == MODE_FULL && n == kRegRows && (!has_last || nlast == kRegRows) && !A.check_finite &&
-        ((reinterpret_cast<uintptr_t>(A.F + (int64_t)blockIdx.y * A.ldf + off + row_lo) |
-          reinterpret_cast<uintptr_t>(A.x + (int64_t)blockIdx.y * A.ldx + off + row_lo) |
-          (ADJ ? reinterpret_cast<uintptr_t>(A.xf + off + row_lo) : (uintptr_t)0)) & 15u) == 0u) {
+    // 16-row blocks, all of full size: the register path
+    if (A.reg_path && A.mode == MODE_FULL && n == kRegRows && (!has_last || nlast == kRegRows) && !A.check_finite) {
       window_reg<NT, ADJ>(A, pp, tab, P, wlo, nwin, hl, nown, row_lo, reinterpret_cast<unsigned char*>(sm));
       return;
     }

@@ -3,10 +3,10 @@
 // A window whose blocks all have 16 rows, whose right-hand side and solution are 16-byte aligned
 // device memory and whose launch asks for the full solve (MODE_FULL, forward) is solved with a
 // thread's pair of blocks (2 x 16 unknowns) kept in registers from the load to the store:
-//   - the window's rows of F arrive by bulk asynchronous copies (cp.async.bulk: one per thread, its
-//     two blocks, 256 contiguous bytes) into shared-memory slots of 272 bytes (the pair plus 16
-//     bytes of padding, so that the per-thread 16-byte reads of eight consecutive threads fall in
-//     eight different bank groups); one mbarrier counts the bytes, its wait is bounded;
+//   - the window's rows of F arrive by 16-byte cp.async copies (8-byte ones where F is not 16-byte
+//     aligned), consecutive threads copying consecutive elements, into shared-memory slots of 272
+//     bytes, one per thread (its two blocks, 256 contiguous bytes, plus 16 bytes of padding, so that
+//     the per-thread 16-byte reads of eight consecutive threads fall in eight different bank groups);
 //   - the exponent range of the window (its power-of-two scale), the split into float-float, the
 //     two constant-coefficient recurrences (a1), the block-end quantities, beta (eq. 16) and the
 //     dichotomy tree (a2, shared with the shared-memory path), the spike correction of eq. 7 (a3)
@@ -14,21 +14,20 @@
 //   - the output scale g = -1/q is folded into the join: the backward recurrence leaves X with
 //     x = g X, the spike correction works in units of X (its coefficients times 1/g = -q), and each
 //     output is one FP64 FMA, g * hi + (g * lo), with the window scale undone in the exponent bits;
-//   - the solution goes back through the same shared-memory slots, and each thread's own (non-halo)
-//     blocks leave by bulk copies to global memory.
-// Windows of any other shape, the adjoint and the general path's passes take the shared-memory
-// path of window_mixed.cuh.  Included by window_mixed.cuh after the tree (tree2, Recs2).
+//   - the solution goes back through the same shared-memory slots, and the window's own (non-halo)
+//     rows leave with coalesced stores.
+// Windows of any other shape and the general path's passes take the shared-memory path of
+// window_mixed.cuh.  Included by window_mixed.cuh after the tree (tree2, Recs2).
 #pragma once
 #include <type_traits>
 #include "ff.cuh"
+#include "slots.cuh"
 #include "window.cuh"
 
 namespace dich {
 
 struct Recs2;
 
-constexpr int kRegRows = 16;                            // block size of the register path
-constexpr int kRegPairBytes = 2 * kRegRows * 8 + 16;    // a thread's two blocks + 16 bytes of padding
 // the middle record's float-float entries a window copies to shared memory at its start (the
 // per-system tables of a batch are then read once per CTA, not at first touch inside the tree): the
 // block-coefficient record, the four beta coefficients and the 66 pair-map powers
@@ -36,55 +35,12 @@ constexpr int kMidRec = 0, kMidK = 10, kMidPow = 14, kMidEntries = 80;
 
 // shared memory of the register path for NT threads: the pair slots, the two spike tables, the
 // warp-boundary first/last values, the scan scratch, the exponent maxima (of the right-hand side
-// and, for the adjoint, of the forward solution), the middle record's entries and the mbarrier
+// and, for the adjoint, of the forward solution) and the middle record's entries
 __host__ __device__ inline size_t window_reg_smem_bytes(int NT) {
   const size_t nw = (size_t)(NT / 32);
   return (size_t)NT * kRegPairBytes + 2 * 16 * (size_t)kRegRows + 8 * 2 * nw + 8 * 4 * nw + 4 * 4 * nw +
-         8 * (size_t)kMidEntries + 16;
+         8 * (size_t)kMidEntries;
 }
-
-// ---------------------------------------------------------------- mbarrier and bulk copies (PTX)
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long* bar, unsigned bytes) {
-  unsigned long long state;
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;"
-               : "=l"(state)
-               : "r"(smem_addr(bar)), "r"(bytes)
-               : "memory");
-  (void)state;
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0u;
-}
-// global -> shared, completion counted in bytes on the mbarrier (16-byte aligned, size a multiple of 16)
-__device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_addr(sdst)),
-               "l"(gsrc), "r"(bytes), "r"(smem_addr(bar))
-               : "memory");
-}
-// shared -> global in the thread's bulk group
-__device__ __forceinline__ void bulk_store(void* gdst, const void* ssrc, unsigned bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst), "r"(smem_addr(ssrc)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// the thread's bulk stores have read their shared-memory source (the CTA may then exit)
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// generic-proxy writes to shared memory become visible to the bulk copies issued after this fence
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // a float's bits rebuilt as an FP64 bit pattern with the exponent rebias k (fast windows, ff.cuh)
 __device__ __forceinline__ double f32_as_f64(float f, unsigned k) {
@@ -197,14 +153,10 @@ __device__ __forceinline__ void tree_mid(const float2* tf, int rm, int pw, const
   if (b1 + 1 < nwin) XR1 = xs_next;
 }
 
-// Iterations of the bounded wait for the window's bulk loads (each try_wait may also suspend the
-// thread for a while); running out latches ST_TIMEOUT and the CTA returns without a store.
-constexpr int kBulkWaitIters = 1 << 22;
-
 // ADJ: the adjoint (a5) -- A.F is w, the plan the transposed one, A.x receives lambda, and the
 // gradient sums -(sum lambda_r x_{r-1}, sum lambda_r x_r, sum lambda_r x_{r+1}) over the window's own
 // rows go to A.part (three per CTA).  The forward solution x (A.xf) comes into the pair slots by a
-// second bulk copy as soon as w has moved to registers, and is read back row by row as lambda is
+// second copy as soon as w has moved to registers, and is read back row by row as lambda is
 // written over it.
 template <int NT, bool ADJ = false>
 __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, const double* tab, int64_t P,
@@ -221,7 +173,6 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
   unsigned* sexp = reinterpret_cast<unsigned*>(swv + 4 * NW);                    // 2 NW exponent maxima
   unsigned* sexpx = sexp + 2 * NW;                                               // the same for x
   float2* mt = reinterpret_cast<float2*>(sexpx + 2 * NW);                        // middle record entries
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(mt + kMidEntries);
 
   const int b0 = 2 * tid, b1 = b0 + 1;
   const bool act0 = b0 < nwin, act1 = b1 < nwin;
@@ -230,15 +181,9 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
   const double* src = A.F + (int64_t)blockIdx.y * A.ldf + pp->off + row_lo;
   double* dst = A.x + (int64_t)blockIdx.y * A.ldx + pp->off + row_lo;
 
-  // ---------------------------------------------------------------- F -> the pair slots (bulk, async)
-  if (tid == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-  if (tid == 0) mbar_arrive_expect_tx(bar, (unsigned)(nwin * R * 8));
-  const unsigned mybytes = (act1 ? 2u : (act0 ? 1u : 0u)) * R * 8u;
-  if (mybytes) bulk_load(mine, src + (int64_t)b0 * R, mybytes, bar);
+  const bool al_src = (reinterpret_cast<uintptr_t>(src) & 15u) == 0u, al_dst = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0u;
+  // ---------------------------------------------------------------- F -> the pair slots (async)
+  slots_load(smem, src, nwin * R, al_src, lane, wid);
   if constexpr (!ADJ) {   // (the adjoint, at four CTAs per SM, reads them from the tables: measured faster)
     const float2* tf = reinterpret_cast<const float2*>(tab);
     for (int i = tid; i < kMidEntries; i += NT) {
@@ -253,12 +198,8 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     tv4[tid] = make_float4(v.x, v.x, v.y, v.y);
     tw4[tid] = make_float4(w.x, w.x, w.y, w.y);
   }
-  bool arrived = false;
-  for (int it = 0; it < kBulkWaitIters && !arrived; ++it) arrived = mbar_try_wait(bar, 0u);
-  if (!__syncthreads_and(arrived)) {
-    if (tid == 0) atomicOr(A.status, (unsigned)ST_TIMEOUT);
-    return;
-  }
+  cp_async_wait_all();
+  __syncwarp();   // (the tables staged above are read after the exponent range's barrier)
 
   // ---------------------------------------------------------------- the pair in registers
   // a[k] = rows 2k, 2k+1 of block 2t; b[k] the same of block 2t+1.  The slot part of an inactive
@@ -311,10 +252,10 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     hlo = (unsigned)(emax - 119) << 20;
   }
   if constexpr (ADJ) {
-    // the slot's values are in registers: it now takes the forward solution x (mbarrier phase 1)
-    fence_async_smem();
-    if (tid == 0) mbar_arrive_expect_tx(bar, (unsigned)(nwin * R * 8));
-    if (mybytes) bulk_load(mine, A.xf + pp->off + row_lo + (int64_t)b0 * R, mybytes, bar);
+    // every thread's slot is in its registers (the barrier of the exponent range): the slots now take
+    // the forward solution x
+    const double* xsrc = A.xf + pp->off + row_lo;
+    slots_load(smem, xsrc, nwin * R, (reinterpret_cast<uintptr_t>(xsrc) & 15u) == 0u, lane, wid);
   }
 
   // fast windows: the FP64 multiplier of the join, G = g 2^(896 - wscale), folds the rebias of the
@@ -410,8 +351,7 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     // ------------------------------------------------------------ correction (a3), join, store
     const bool own0 = act0 && b0 >= hl && b0 < hl + nown;
     const bool own1 = act1 && b1 >= hl && b1 < hl + nown;
-    if (!ADJ && !(own0 || own1)) return;
-    const bool anyown = ADJ ? (own0 || own1) : true;   // forward: every thread past here owns a block
+    const bool anyown = own0 || own1;
     // x = xp + (x_{s-1} - xp(-1)) v + x_{e+1} w, in units of X (x = g X; the tree's first/last values
     // are in those units already): the coefficients are X_{s-1} - ib X_0 and X_{e+1}
     const ff2 ibx = ff2_mul(ff2_bcast(ffv{pp->ib_h, pp->ib_l}), X0);
@@ -425,12 +365,8 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     bool xfast = false;
     double xlb = 0.0, xrb = 0.0;
     if constexpr (ADJ) {
-      bool got = false;
-      for (int it = 0; it < kBulkWaitIters && !got; ++it) got = mbar_try_wait(bar, 1u);
-      if (!__syncthreads_and(got)) {
-        if (tid == 0) atomicOr(A.status, (unsigned)ST_TIMEOUT);
-        return;
-      }
+      cp_async_wait_all();
+      __syncthreads();
       unsigned hmax = 0u, hmin = 0xFFFFFFFFu;
 #pragma unroll
       for (int k = 0; k < R / 2; ++k) {
@@ -507,6 +443,7 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     // way (half the code: measured 2.8% faster, the instruction cache then missing less); the
     // adjoint's rows are in registers
     constexpr int KUNROLL = ADJ ? R / 2 : 4;
+    if (ADJ || anyown)   // forward: the halo's rows are not wanted
 #pragma unroll KUNROLL
     for (int k = 0; k < R / 2; ++k) {
       double o0[2], o1[2];
@@ -589,16 +526,8 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
         xb = nb2;
       }
     }
-    if (anyown) {
-      fence_async_smem();
-      if (own0 && own1)
-        bulk_store(dst + (int64_t)b0 * R, mine, 2u * R * 8u);
-      else if (own0)
-        bulk_store(dst + (int64_t)b0 * R, mine, R * 8u);
-      else
-        bulk_store(dst + (int64_t)b1 * R, mine + 8 * R, R * 8u);
-      bulk_commit();
-    }
+    __syncwarp();   // the warp's rows of x are in its slots
+    slots_store(smem, dst, hl * R, (hl + nown) * R, al_dst, lane, wid);
     if constexpr (ADJ) {
       // the CTA's three sums: the thread's own lanes, the warp, the CTA (fixed order), one join
       __syncthreads();   // the scan scratch takes the per-warp sums
@@ -646,7 +575,6 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
       store_loop(std::true_type());
     else
       store_loop(std::false_type());
-    if (anyown) bulk_wait_read();
   };
   if (fast && gfold)
     body(std::true_type(), std::true_type(), std::false_type());
