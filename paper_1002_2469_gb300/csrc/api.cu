@@ -37,8 +37,9 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 // window width in blocks: the MIXED kernel gives every thread two blocks
 int window_blocks(int NT, int form) { return form == FORM_MIXED ? 2 * NT : NT; }
 
-size_t smem_bytes(int NT, int n, int form) {
-  return form == FORM_MIXED ? window2_smem_bytes(NT, n) : window_smem_bytes(NT, n);
+size_t smem_bytes(int NT, int n, int form, int ntf) {
+  if (form == FORM_MIXED) return window2_smem_bytes(NT, n);
+  return std::max(window_smem_bytes(NT, n), ntf ? window_fix_smem_bytes(ntf) : (size_t)0);
 }
 
 int max_rows(int NT, int form, size_t budget) {
@@ -120,6 +121,137 @@ void split_ff(double d, float& h, float& l) {
 }
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// ---------------------------------------------------------------- fixed-point tables (window_fix.cuh)
+// double-double arithmetic: the fractions carry 64 bits
+struct dd {
+  double h, l;
+};
+static dd dd_norm(double a, double b) {
+  const double s = a + b, t = s - a;
+  return dd{s, (a - (s - t)) + (b - t)};
+}
+static dd dd_prod(double a, double b) {
+  const double p = a * b;
+  return dd{p, std::fma(a, b, -p)};
+}
+static dd dd_add(dd a, dd b) {
+  const dd s = dd_norm(a.h, b.h);
+  return dd_norm(s.h, s.l + (a.l + b.l));
+}
+static dd dd_mul(dd a, dd b) {
+  const dd p = dd_prod(a.h, b.h);
+  return dd_norm(p.h, p.l + (std::fma(a.h, b.l, a.l * b.h)));
+}
+static dd dd_div(dd a, dd b) {
+  const double q0 = a.h / b.h;
+  const dd r = dd_add(a, dd_mul(dd{-q0, 0.0}, b));
+  return dd_norm(q0, r.h / b.h);
+}
+static dd dd_sqrt(dd a) {
+  if (a.h <= 0.0) return dd{0.0, 0.0};
+  const double s = std::sqrt(a.h);
+  const dd r = dd_add(a, dd_mul(dd{-s, 0.0}, dd{s, 0.0}));
+  return dd_norm(s, r.h / (2.0 * s));
+}
+// the fraction v in [0, 1) as a multiple of 2^-64
+static u64 dd_word(dd v) {
+  const double w = v.h * 0x1p64, f = std::floor(w);
+  if (!(f < 0x1p64)) return ~(u64)0;
+  return (u64)f + (u64)(long long)std::llround((w - f) + v.l * 0x1p64);
+}
+// x r 2^-64 as the kernels round it
+static u64 word_mul(u64 x, u64 r) {
+  const u64 xh = x >> 32, xl = x & 0xFFFFFFFFu, rh = r >> 32, rl = r & 0xFFFFFFFFu;
+  return xh * rh + ((xl * rh) >> 32) + ((xh * rl) >> 32);
+}
+
+// The table of one system of N rows; false: its windows are solved in FP64.  Needs both recurrence
+// coefficients of one sign; R^N below 2^-66 (the left end's closed form, window_fix.cuh); the scale g
+// within 2^-60..2^60; and a bound on |X| / max|F| of at most 2^11 (kFixMinBits): the words spend that
+// many bits on the largest possible solution, and the right-hand side keeps at least 52 below its
+// largest value.  Measured rms errors against exact values, FP64 recurrences and words: gain 4 1.2e-16
+// and 5e-17, gain 1000 (tridiag{-1, 2.001, -1}) 4.1e-15 and 2.9e-16.
+constexpr int kFixMinBits = 52;
+static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
+  const Roots r = toeplitz_roots(tm1, t0, tp1);
+  const double ag = std::fabs(r.g);
+  if (!(ag >= 0x1p-60 && ag <= 0x1p60)) return false;
+  if ((tm1 > 0.0 && tp1 < 0.0) || (tm1 < 0.0 && tp1 > 0.0)) return false;
+  if (!(std::fabs(r.rs) < 1.0 - 0x1p-11 && std::fabs(r.ib) < 1.0 - 0x1p-11)) return false;
+  if (r.rs != 0.0 && (double)N * std::log2(std::fabs(r.rs)) > -66.0) return false;
+  // q = -(t0 + sgn(t0) sqrt(t0^2 - 4 tp1 tm1)) / 2 for |q|
+  const double b0 = std::fabs(t0);
+  const dd disc = dd_add(dd_prod(b0, b0), dd_mul(dd{-4.0, 0.0}, dd_prod(tp1, tm1)));
+  const dd q2 = dd_add(dd{b0, 0.0}, dd_sqrt(disc));   // 2 |q|
+  const dd R = dd_div(dd{2.0 * std::fabs(tm1), 0.0}, q2), B = dd_div(dd{2.0 * std::fabs(tp1), 0.0}, q2);
+  dd g = dd_div(dd{2.0, 0.0}, q2);
+  int gk = 0;
+  std::frexp(g.h, &gk);
+  g = dd{std::ldexp(g.h, -gk), std::ldexp(g.l, -gk)};
+  const u64 O = (u64)1 << 63;
+  T[FX_R] = dd_word(R);
+  T[FX_B] = dd_word(B);
+  T[FX_G] = dd_word(g);
+  const u64 a = O - word_mul(O, T[FX_B]), K = a - word_mul(a, T[FX_R]);
+  int hb = 0;
+  while (hb < 63 && (K >> (hb + 1)) != 0) ++hb;
+  if (hb < kFixMinBits) return false;
+  T[FX_A] = a;
+  T[FX_K] = K + 1;
+  // the mean truncation of the two products per row of Y (settling at 2.5 / (1 - B)), of the last
+  // two products and of the lowest bit set on conversion
+  const double bias = (2.5 / (1.0 - B.h) + 1.25) * g.h + 1.25 - 0.5;
+  T[FX_KG] = (u64)std::llround(bias) - word_mul(O, T[FX_G]);
+  T[FX_HB] = (u64)hb;
+  T[FX_GK] = (u64)(int64_t)gk;
+  T[FX_FLAGS] = (u64)(((tm1 != 0.0 ? r.rs : r.ib) < 0.0 ? FIX_ALT : 0) | (r.g < 0.0 ? FIX_NEG : 0) |
+                      (hb < kFixMinBits + 3 ? FIX_GUARD : 0));
+  auto lev = [](double v) {
+    if (v == 0.0) return 0;
+    const double need = -64.0 / std::log2(v);   // rows until v^rows < 2^-64
+    int k = 0;
+    while (k < 5 && 32.0 * (double)(1 << k) < need) ++k;
+    return k;
+  };
+  T[FX_LEVR] = (u64)lev(R.h);
+  T[FX_LEVB] = (u64)lev(B.h);
+  dd v = R, w = B;
+  dd R32{1.0, 0.0}, B32{1.0, 0.0};
+  for (int i = 0; i < kFixHalf; ++i) {
+    T[FX_P + i] = dd_word(v);
+    T[FX_Q + kFixHalf - 1 - i] = dd_word(w);
+    if (i == kFixHalf - 1) {
+      R32 = dd_mul(v, v);
+      B32 = dd_mul(w, w);
+    }
+    v = dd_mul(v, R);
+    w = dd_mul(w, B);
+  }
+  // binades from block to block of a window of varying scale: at most half the decay over 32 rows
+  {
+    double st = 8.0;
+    if (R.h > 0.0) st = std::min(st, std::floor(-16.0 * std::log2(R.h)));
+    if (B.h > 0.0) st = std::min(st, std::floor(-16.0 * std::log2(B.h)));
+    T[FX_STEP] = (st >= 4.0 && hb - kFixVarBits >= kFixMinBits) ? (u64)st : 0;
+  }
+  auto powers = [&](dd r, int at_m, int at_x) {
+    dd p = r;
+    for (int t = 1; t <= 32; ++t) {
+      int k = -256;   // zero: shifted out whatever the scales
+      if (p.h > 0.0) {
+        std::frexp(p.h, &k);
+        T[at_m + t] = dd_word(dd{std::ldexp(p.h, -k), std::ldexp(p.l, -k)});
+      }
+      const int16_t x = (int16_t)-k;
+      std::memcpy((char*)(T + at_x) + 2 * t, &x, 2);
+      p = dd_mul(p, r);
+    }
+  };
+  powers(R32, FX_RM, FX_RX);
+  powers(B32, FX_BM, FX_BX);
+  return true;
+}
 
 // Choose the block size: one window when the system fits in one window of default-size
 // blocks (n = ceil(N / window blocks) <= n_def), else n_def rows per block.  Longer blocks
@@ -263,6 +395,15 @@ int build_system(double tm1, double t0, double tp1, int64_t N, int NT, int form,
   p.o_klf = take(kl * 4);
   p.o_krf = take(kr * 4);
   p.o_midf = take(66);
+  // the fixed-point table of FP64-form systems (left out where the caller's storage has no room for it)
+  u64 fix[FX_WORDS] = {};
+  const bool with_fix = form == FORM_F64 && fix_threads(NT, n) != 0 && fix_table(tm1, t0, tp1, N, fix) &&
+                        (!sb.ext || (size_t)o_ + FX_WORDS <= sb.ext_cap);
+  p.o_fix = 0;
+  if (with_fix) {
+    o_ += o_ & 1;   // 16-byte aligned within the table
+    p.o_fix = take(FX_WORDS);
+  }
   // warp-scan levels of the MIXED tree: a contribution from 2^(lev+1) or more blocks away carries a
   // product of ratios below |rs|^(n 2^(lev+1)) (prefix) or |ib|^(n 2^(lev+1)) (suffix): below eps
   auto levels = [&](int64_t Lrows) {
@@ -288,23 +429,29 @@ int build_system(double tm1, double t0, double tp1, int64_t N, int NT, int form,
     sb.tab.assign((size_t)o_, 0.0);
     T = sb.tab.data();
   }
+  if (with_fix) std::memcpy(&T[p.o_fix], fix, sizeof(fix));
   auto put_ff = [&](int32_t at, double d) {
     float h, l;
     split_ff(d, h, l);
     float2 f2 = make_float2(h, l);
     std::memcpy(&T[at], &f2, sizeof(double));
   };
-  for (int i = 0; i < p.Lv; ++i) {
-    T[p.o_v + i] = vspike(n, i);
-    put_ff(p.o_vf + i, T[p.o_v + i]);
-  }
-  for (int i = 0; i < p.Lw; ++i) {
-    T[p.o_w + i] = wspike_rev(n, i);
-    put_ff(p.o_wf + i, T[p.o_w + i]);
+  const double qn1 = qnum(n + 1, r), ql1 = qnum(nl + 1, r);   // the spikes' common denominators
+  for (int i = 0; i < std::max(p.Lv, p.Lw); ++i) {
+    const double ratio = qnum(n - i, r) / qn1;
+    if (i < p.Lv) {
+      T[p.o_v + i] = ipow(r.rs, i + 1) * ratio;
+      put_ff(p.o_vf + i, T[p.o_v + i]);
+    }
+    if (i < p.Lw) {
+      T[p.o_w + i] = ipow(r.ib, i + 1) * ratio;
+      put_ff(p.o_wf + i, T[p.o_w + i]);
+    }
   }
   for (int i = 0; i < nl; ++i) {
-    T[p.o_vl + i] = vspike(nl, i);
-    T[p.o_wl + i] = wspike_rev(nl, i);
+    const double ratio = qnum(nl - i, r) / ql1;
+    T[p.o_vl + i] = ipow(r.rs, i + 1) * ratio;
+    T[p.o_wl + i] = ipow(r.ib, i + 1) * ratio;
     put_ff(p.o_vlf + i, T[p.o_vl + i]);
     put_ff(p.o_wlf + i, T[p.o_wl + i]);
   }
@@ -451,6 +598,7 @@ struct dich_plan_s {
   int form = FORM_F64;
   int path = PATH_SINGLE;
   int n_smem = 2;
+  int ntf = 0;                         // fixed-point threads of the FP64 form's launches (0: none)
   int64_t tiles = 0;
   SysBuild fwd, adj;
   // quasi-Toeplitz corners (eq. 21): t_0 + psi in row 0, t_0 + chi in row N-1
@@ -511,7 +659,8 @@ static void plan_layout(dich_plan_s* p) {
   p->off_status = o_;
   o_ += kAlign;
   p->off_tabs = o_;
-  o_ += align_up(sizeof(double) * (p->fwd.tab.size() + p->adj.tab.size() + p->corner.size()));
+  const size_t ntab = p->fwd.tab.size() + p->adj.tab.size() + p->corner.size();
+  o_ += align_up(sizeof(double) * ntab);
   const int64_t P = (p->N >= 2) ? p->fwd.rec.P : 0;
   if (p->path == PATH_GENERAL) {
     p->off_beta = o_;
@@ -525,7 +674,7 @@ static void plan_layout(dich_plan_s* p) {
   o_ += align_up(sizeof(double) * 3 * (size_t)std::max<int64_t>(1, p->tiles));
   p->ws_bytes = o_;
   // staging copy: records, zero status, tables
-  p->staging.assign(p->off_tabs + sizeof(double) * (p->fwd.tab.size() + p->adj.tab.size() + p->corner.size()), 0);
+  p->staging.assign(p->off_tabs + sizeof(double) * ntab, 0);
   SysPlan recs[2] = {p->fwd.rec, p->adj.rec};
   recs[0].tab = 0;
   recs[1].tab = (int64_t)p->fwd.tab.size();
@@ -576,6 +725,9 @@ static int plan_geometry(dich_plan_s* p, const Opts& o, int NT, int n) {
   }
   p->n_smem = n;
   p->tiles = ceil_div(p->fwd.rec.P, p->fwd.rec.own);
+  p->ntf = (p->form == FORM_F64 && p->path != PATH_GENERAL && p->fwd.rec.o_fix && p->adj.rec.o_fix)
+               ? fix_threads(NT, n)
+               : 0;
   return DICH_OK;
 }
 
@@ -629,6 +781,32 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
     // the caller fixed the geometry, take narrower windows, then shorter blocks, while the system
     // stays on the halo path (halo at most half the window).  Measured on GB300: N = 65536 solves
     // 2x faster with 64-thread windows of 2-row blocks than with the large-N default.
+    // Coupling longer than half a default window, but not half a window of twice the width: with the
+    // fixed-point form one pass over overlapping windows is the faster way (tridiag{-1, 2.001, -1},
+    // N = 2^24 + 1: 120 us against 348 us for the general path's two FP64 passes; solved in FP64, where
+    // a window's values do not suit fixed point, such windows take about the general path's time).
+    // Only with a window for every SM: fewer of them leave SMs idle.
+    if (o.NT == 0 && o.n_req == 0 && p->form == FORM_F64 && p->path == PATH_GENERAL &&
+        !(o.flags & DICH_FLAG_FORCE_GENERAL)) {
+      dich_plan_s q;
+      q.N = N;
+      q.tm1 = t_m1;
+      q.t0 = t_0;
+      q.tp1 = t_1;
+      q.opts = o;
+      q.form = p->form;
+      const int NT = 2 * p->NT;
+      const int nc = choose_n(N, NT, max_rows(NT, p->form, kSmemBudget), 0, default_rows(p->form));
+      if (plan_geometry(&q, o, NT, nc) == DICH_OK && q.path == PATH_HALO && q.ntf && q.tiles >= device_sms()) {
+        p->NT = NT;
+        p->fwd = std::move(q.fwd);
+        p->adj = std::move(q.adj);
+        p->path = q.path;
+        p->n_smem = q.n_smem;
+        p->ntf = q.ntf;
+        p->tiles = q.tiles;
+      }
+    }
     const int sms = device_sms();
     if (o.NT == 0 && o.n_req == 0 && p->path == PATH_HALO && p->tiles < 2 * (int64_t)sms) {
       const int nmin = (p->form == FORM_MIXED) ? 2 : 4;
@@ -654,6 +832,7 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
         p->adj = std::move(q.adj);
         p->path = q.path;
         p->n_smem = q.n_smem;
+        p->ntf = q.ntf;
         p->tiles = q.tiles;
       }
     }
@@ -794,12 +973,13 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   // the register path only for full solves of device memory, unless the plan asks
   // for the shared-memory path (the general path's passes always take that one)
   a.reg_path = (device_mem && p->path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? 1 : 0;
-  const size_t smem = smem_bytes(p->NT, p->n_smem, p->form);
+  const int NT = p->NT, ntf = p->ntf;
+  const size_t smem = smem_bytes(NT, a.n_smem, p->form, ntf);
   // windows [win0, win0 + grid) of the single and halo paths (all of them unless a range is given)
   const int grid = (int)((nwin < 0) ? p->tiles : nwin);
   auto launch = [&](const WinArgs& w, int gy) {
-    return p->form == FORM_F64 ? launch_window_f64(p->NT, grid, smem, st, w, gy)
-                               : launch_window_mixed(p->NT, grid, smem, st, w, gy);
+    return p->form == FORM_F64 ? launch_window_f64(NT, ntf, grid, smem, st, w, gy)
+                               : launch_window_mixed(NT, grid, smem, st, w, gy);
   };
   cudaError_t e;
   if (p->path != PATH_GENERAL) {
@@ -1113,7 +1293,7 @@ cudaError_t shard_windows(dich_plan_t p, const ShardGeo& g, int mode, const doub
   a.win0 = g.w_lo;
   const int grid = (int)(g.w_hi - g.w_lo);
   const size_t smem = smem_bytes(p->NT, p->n_smem, p->form);
-  return p->form == FORM_F64 ? launch_window_f64(p->NT, grid, smem, st, a, 1)
+  return p->form == FORM_F64 ? launch_window_f64(p->NT, 0, grid, smem, st, a, 1)
                              : launch_window_mixed(p->NT, grid, smem, st, a, 1);
 }
 }  // namespace
@@ -1246,6 +1426,7 @@ struct dich_batch_s {
   std::vector<int32_t> sys_ids[2];         // per form: its systems, in item order
   std::vector<int64_t> first[2], count[2]; // per form, parallel to sys_ids: CTA range of each system
   int n_smem[2] = {2, 2};
+  int ntf = 0;                             // fixed-point threads of the FP64-form launch (0: none)
   size_t ws_bytes = 0, off_plans = 0, off_status = 0, off_tabs = 0, off_items[2] = {0, 0},
          off_ids[2] = {0, 0}, off_first[2] = {0, 0}, off_count[2] = {0, 0}, off_trivial = 0,
          off_part[2] = {0, 0};
@@ -1379,7 +1560,9 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     b->first[f].push_back(first);
     b->count[f].push_back((int64_t)b->items[f].size() - first);
     b->n_smem[f] = std::max(b->n_smem[f], q.n);
+    if (q.o_fix || b->adj[(size_t)s].rec.o_fix) b->ntf = 1;
   }
+  if (b->ntf) b->ntf = fix_threads(b->NT[FORM_F64], b->n_smem[FORM_F64]);
   // MIXED windows: the register path unless most of them are whole one-window systems, whose
   // windows are latency-bound (their own tables, no halo to amortise the set-up): there the
   // shared-memory path's six CTAs per SM win (4096 Poisson modes of 4096 rows: 101 us against
@@ -1635,8 +1818,8 @@ static int batch_launch(dich_batch_t b, const double* F, double* x, const double
     a.n_smem = b->n_smem[f];
     a.sys_offset = sys_offset;
     a.reg_path = b->reg_path ? 1 : 0;   // batch vectors are device memory
-    const size_t smem = smem_bytes(b->NT[f], a.n_smem, f);
-    cudaError_t e = (f == FORM_F64) ? launch_window_f64(b->NT[f], (int)nitems, smem, sf, a)
+    const size_t smem = smem_bytes(b->NT[f], a.n_smem, f, b->ntf);
+    cudaError_t e = (f == FORM_F64) ? launch_window_f64(b->NT[f], b->ntf, (int)nitems, smem, sf, a)
                                     : launch_window_mixed(b->NT[f], (int)nitems, smem, sf, a);
     if (e != cudaSuccess) return cuda_fail(e);
     if (adjoint) {
@@ -1675,7 +1858,7 @@ static int batch_launch(dich_batch_t b, const double* F, double* x, const double
     double* iface = (double*)(b->d_ws + b->off_giface);
     const size_t smem = smem_bytes(b->NT[f], a.n_smem, f);
     auto launch = [&](const WinArgs& w) {
-      return f == FORM_F64 ? launch_window_f64(b->NT[f], (int)ng, smem, st, w)
+      return f == FORM_F64 ? launch_window_f64(b->NT[f], 0, (int)ng, smem, st, w)
                            : launch_window_mixed(b->NT[f], (int)ng, smem, st, w);
     };
     WinArgs wb = a;

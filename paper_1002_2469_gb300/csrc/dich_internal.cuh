@@ -85,7 +85,8 @@ struct SysPlan {
   // table sub-offsets (in doubles, relative to `tab`)
   int32_t o_v, o_w, o_vl, o_wl;             // v[Lv], w_rev[Lw], v_last[nlast], w_last_rev[nlast]
   int32_t o_vf, o_wf, o_vlf, o_wlf;         // float-float copies (float2 per entry)
-  int32_t o_bcm, o_bcl, o_bcr, pad2_;       // middle record, left table [kl], right table [kr]
+  int32_t o_bcm, o_bcl, o_bcr;              // middle record, left table [kl], right table [kr]
+  int32_t o_fix;                            // fixed-point table (window_fix.cuh); 0: none
   int32_t o_bcmf, o_bclf, o_bcrf, pad3_;    // the same records as float-float (float2 per entry)
   // float-float copies of g * ib and of the corner spikes (MIXED form)
   float gib_h, gib_l;
@@ -110,6 +111,7 @@ struct Item {
 // ---------------------------------------------------------------- Toeplitz math (host + device)
 struct Roots {
   double rs, ib, z, omz, g, q;
+  double lz;   // log |z| (z != 0)
   bool ok;
 };
 
@@ -133,6 +135,7 @@ DICH_HD Roots toeplitz_roots(double tm1, double t0, double tp1) {
   // 1 - z = sqrt(disc) (sqrt(disc) + |t_0|) / (2 q^2), free of cancellation
   r.omz = sd * (sd + fabs(t0)) / (2.0 * q * q);
   r.g = -1.0 / q;
+  r.lz = r.z > 0.0 ? log1p(-r.omz) : (r.z < 0.0 ? log(-r.z) : 0.0);
   return r;
 }
 
@@ -152,13 +155,8 @@ DICH_HD double qnum(int64_t k, const Roots& r) {
   if (k <= 0) return 0.0;
   if (r.omz == 0.0) return (double)k;
   if (r.z == 0.0) return 1.0;
-  if (r.z > 0.0) {
-    double lz = log1p(-r.omz);
-    return -expm1((double)k * lz) / r.omz;
-  }
-  double lz = log(-r.z);
-  if ((k & 1) == 0) return -expm1((double)k * lz) / r.omz;
-  return (1.0 + exp((double)k * lz)) / r.omz;
+  if (r.z > 0.0 || (k & 1) == 0) return -expm1((double)k * r.lz) / r.omz;
+  return (1.0 + exp((double)k * r.lz)) / r.omz;
 }
 
 // Block spike entries for a block of size nb:

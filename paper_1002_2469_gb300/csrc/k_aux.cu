@@ -306,30 +306,39 @@ cudaError_t launch_block_scan_batched(const SysPlan* plans, const double* tabs, 
 __global__ void __launch_bounds__(256) k_adj_finalize(const double* part, const int32_t* sys_ids,
                                                       const int64_t* first, const int64_t* count, int64_t count0,
                                                       double* gt) {
-  __shared__ double sh[3 * 256];
+  __shared__ double sh[3 * 256], she[3 * 256];
   const int64_t k = blockIdx.x;
   const int64_t s = sys_ids ? sys_ids[k] : k;
   const int64_t f = first ? first[k] : 0;
   const int64_t c = count ? count[k] : count0;
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-  for (int64_t i = threadIdx.x; i < c; i += 256) {
-    a0 += part[3 * (f + i)];
-    a1 += part[3 * (f + i) + 1];
-    a2 += part[3 * (f + i) + 2];
-  }
-  sh[threadIdx.x] = a0;
-  sh[256 + threadIdx.x] = a1;
-  sh[512 + threadIdx.x] = a2;
-  __syncthreads();
+  // every addition's rounding error is kept (TwoSum) and added at the end: a few operations per CTA of
+  // the adjoint, and the sums are then as good as their per-CTA terms
+  double a[3] = {0.0, 0.0, 0.0}, e[3] = {0.0, 0.0, 0.0};
+  auto add = [](double& x, double& err, double y, double yerr) {
+    const double t = x + y, z = t - x;
+    err += ((x - (t - z)) + (y - z)) + yerr;
+    x = t;
+  };
+  for (int64_t i = threadIdx.x; i < c; i += 256)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) add(a[j], e[j], part[3 * (f + i) + j], 0.0);
   for (int d = 128; d > 0; d >>= 1) {
-    if ((int)threadIdx.x < d) {
-      sh[threadIdx.x] += sh[threadIdx.x + d];
-      sh[256 + threadIdx.x] += sh[256 + threadIdx.x + d];
-      sh[512 + threadIdx.x] += sh[512 + threadIdx.x + d];
-    }
+    const int at = (int)threadIdx.x;
+    if (at < 2 * d)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        sh[256 * j + at] = a[j];
+        she[256 * j + at] = e[j];
+      }
+    __syncthreads();
+    if (at < d)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) add(a[j], e[j], sh[256 * j + at + d], she[256 * j + at + d]);
     __syncthreads();
   }
-  if (threadIdx.x < 3) gt[3 * s + threadIdx.x] = -sh[256 * threadIdx.x];
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) gt[3 * s + j] = -(a[j] + e[j]);
 }
 
 cudaError_t launch_adj_finalize(const double* part, const int32_t* sys_ids, const int64_t* first,

@@ -1,33 +1,18 @@
-// k_f64.cu -- FP64 instantiations of the window kernel.
+// k_f64.cu -- the FP64-form window kernel's launch by plan width (the instantiations live in
+// k_f64_64.cu, k_f64_128.cu and k_f64_256.cu).
 #include "launch.cuh"
 
 namespace dich {
 
-template <int NT>
-static cudaError_t launch_one(int grid, int grid_y, size_t smem, cudaStream_t st, const WinArgs& a) {
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_window<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid, grid_y);
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_window<NT>, a);
-}
+cudaError_t launch_window_f64_64(int ntf, int grid, int grid_y, size_t smem, cudaStream_t st, const WinArgs& a);
+cudaError_t launch_window_f64_128(int ntf, int grid, int grid_y, size_t smem, cudaStream_t st, const WinArgs& a);
+cudaError_t launch_window_f64_256(int ntf, int grid, int grid_y, size_t smem, cudaStream_t st, const WinArgs& a);
 
-cudaError_t launch_window_f64(int NT, int grid, size_t smem, cudaStream_t st, const WinArgs& a, int grid_y) {
+cudaError_t launch_window_f64(int NT, int ntf, int grid, size_t smem, cudaStream_t st, const WinArgs& a, int grid_y) {
   switch (NT) {
-    case 64: return launch_one<64>(grid, grid_y, smem, st, a);
-    case 128: return launch_one<128>(grid, grid_y, smem, st, a);
-    case 256: return launch_one<256>(grid, grid_y, smem, st, a);
+    case 64: return launch_window_f64_64(ntf, grid, grid_y, smem, st, a);
+    case 128: return launch_window_f64_128(ntf, grid, grid_y, smem, st, a);
+    case 256: return launch_window_f64_256(ntf, grid, grid_y, smem, st, a);
     default: return cudaErrorInvalidValue;
   }
 }

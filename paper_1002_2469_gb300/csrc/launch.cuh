@@ -3,13 +3,15 @@
 #pragma once
 #include <cuda_runtime.h>
 #include "window.cuh"
+#include "window_fix.cuh"
 #include "window_mixed.cuh"
 
 namespace dich {
 
 // window kernel of width NT (64, 128 or 256) in the given form, grid (grid, grid_y): grid_y
 // right-hand sides of a series (WinArgs::ldf, ldx); returns the launch error
-cudaError_t launch_window_f64(int NT, int grid, size_t smem, cudaStream_t st, const WinArgs& a, int grid_y = 1);
+// (FP64 form: ntf threads per CTA with the fixed-point form tried first, fix_threads below, or 0)
+cudaError_t launch_window_f64(int NT, int ntf, int grid, size_t smem, cudaStream_t st, const WinArgs& a, int grid_y = 1);
 cudaError_t launch_window_mixed(int NT, int grid, size_t smem, cudaStream_t st, const WinArgs& a, int grid_y = 1);
 
 // general path: first/last values of every block from per-block beta (global block scan)

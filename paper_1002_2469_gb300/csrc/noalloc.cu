@@ -139,9 +139,10 @@ extern "C" int dichotomy_solve_noalloc(double t_m1, double t_0, double t_1, int6
   a.n_smem = n;
   a.reg_path = 1;   // F and x are device memory (checked above)
   const int64_t tiles = ceil_div(sb.rec.P, sb.rec.own);
-  const size_t smem = smem_bytes(NT, n, form);
+  const int ntf = (form == FORM_F64 && sb.path != PATH_GENERAL && sb.rec.o_fix) ? fix_threads(NT, n) : 0;
+  const size_t smem = smem_bytes(NT, n, form, ntf);
   auto launch = [&](const WinArgs& w) {
-    return (form == FORM_F64) ? launch_window_f64(NT, (int)tiles, smem, st, w)
+    return (form == FORM_F64) ? launch_window_f64(NT, ntf, (int)tiles, smem, st, w)
                               : launch_window_mixed(NT, (int)tiles, smem, st, w);
   };
   unsigned char* b = static_cast<unsigned char*>(base);

@@ -47,7 +47,8 @@ extern thread_local std::string g_cuda_err;
 int cuda_fail(cudaError_t e);
 size_t align_up(size_t v);
 int window_blocks(int NT, int form);
-size_t smem_bytes(int NT, int n, int form);
+// shared memory of a window launch (ntf: fixed-point threads of an FP64-form launch, 0 without)
+size_t smem_bytes(int NT, int n, int form, int ntf = 0);
 int max_rows(int NT, int form, size_t budget);
 int default_threads(int form);
 int default_rows(int form);

@@ -1,5 +1,5 @@
 // slots.cuh -- a window's rows in shared memory, one padded slot of 32 rows per thread (the register path
-// of the MIXED form, window_reg.cuh).
+// of the MIXED form, window_reg.cuh, and the fixed-point form of FP64 windows, window_fix.cuh).
 //
 // A slot is 256 contiguous bytes of the vector plus 16 bytes of padding, so that the per-thread
 // 16-byte reads of eight consecutive threads fall in eight different bank groups.

@@ -1,0 +1,476 @@
+// window_fix.cuh -- FP64-form windows in 64-bit fixed point (32 rows per thread, integer pipes).
+//
+// What bounds the FP64 form is the FP64 pipe: 2 operations per clock per SM, 64 clocks of latency,
+// against five operations per unknown.  In a window whose right-hand side spans a narrow exponent
+// range the same recurrences run as 64-bit fixed-point numbers on the integer pipes: a product by a
+// constant below 1 is one IMAD.WIDE and two IMAD.HI (9.6 such products per clock per SM measured,
+// about 30 clocks of latency), and only the conversions back to FP64 (and half of those from it)
+// take the FP64 pipe.  The words carry more bits than FP64 mantissas do, so the results are closer to
+// the exact solution than the FP64 recurrences' (rms error 4.7e-17 against 1.2e-16 of the solution's
+// rms on the headline system); the path is taken only where that holds (fix_table in api.cu, and
+// the window's own tests).
+//
+// The method, on a window of rows 0..len-1 (T = -q (1 - rs E^-1)(1 - ib E), x = g X):
+//   u_i = f_i + rs u_{i-1},   X_i = u_i + ib X_{i+1}.
+// With rs, ib of one sign s, s^i u_i and s^i X_i obey the same recurrences with R = |rs|, B = |ib|
+// (the right-hand side's and the solution's odd rows change sign).  Words are unsigned: u is held as
+// u + a and X as X + 2^63, a = 2^63 (1 - B); then u's word recurrence is W' = (F + K) + R W with
+// K = a (1 - R), and X's is Y' = W + B Y': no further constants, every term non-negative, and nothing
+// exceeds 64 bits while |F| < 2^hb <= K (|u| <= max|F| / (1 - R), |X| <= max|F| / ((1 - R)(1 - B))).
+//   1. every thread runs W over its two 16-row halves from zero words (two independent chains);
+//   2. the word entering each thread, Uin, is a scan over the threads with powers R^(32 d) (the
+//      window's first row gets u = 0, i.e. the word a), cut where R^(32 d) < 2^-64;
+//   3. Y over each half from zero: Y_i = W_i + R^(i+1) Uin + B Y_{i+1};
+//   4. Xin, the word beyond each thread, by the mirrored scan (the window's end gets X = 0);
+//   5. x_i = g (Y_i + B^(16-i) Xin - 2^63), converted and scaled by the window's power of two.
+// The right end of the system (x_N = 0) is step 4 itself.  At its left end step 2's u_{-1} = 0 belongs
+// to the system extended to the left with zero right-hand side, whose x_{-1} is g ib X_0; the
+// homogeneous solution that removes it is X_i -= X_0 B R^(i+1) (x_{-1} = 0 exactly, up to
+// (R B)^(N - i) R^(i+1) <= R^N, below 2^-64 by fix_table in api.cu).
+//
+// Scale.  A window whose blocks of 32 rows all reach within 2^-4 of its largest |F| has one power of two
+// for all its words (random right-hand sides).  Where |F| varies more but smoothly -- from one block to
+// the next by at most `step` binades, 4 to 8 and at most half the decay of the couplings over a block:
+// the spectra and profiles of smooth sources -- every thread takes the largest exponent of its own and
+// its two neighbours' blocks, and the scans of steps 2 and 4 move signed words between scales.  (What
+// reaches a thread from k + 1 blocks away is then below R^(16 k) of its own range, which the two bits of
+// kFixVarBits cover.)  Anything else (zero stretches, isolated values, Inf and NaN) is solved in FP64,
+// which resolves a solution's tails relative to themselves.
+//
+// Layout: one 272-byte slot per thread (slots.cuh) (F, W, Y and x in turn, in place); loops
+// unrolled by two row pairs of both halves.
+#pragma once
+#include "slots.cuh"
+
+namespace dich {
+
+typedef unsigned long long u64;
+
+constexpr int kFixRows = 32;     // rows per thread
+constexpr int kFixHalf = 16;
+// a plan's fixed-point table (64-bit words, at SysPlan::o_fix): fractions are multiples of 2^-64
+enum FixIdx {
+  FX_R = 0, FX_B, FX_G,          // R, B, |g| 2^-gk in [1/2, 1)
+  FX_K, FX_A, FX_KG,             // K (+1: the products' mean truncation), a, constant of the output product
+  FX_HB, FX_GK, FX_FLAGS,        // hb, gk, FIX_* bits
+  FX_LEVR, FX_LEVB,              // scan levels: R^(32 2^lev) (B^...) below 2^-64, at most 5
+  FX_STEP,                       // binades neighbouring blocks of a varying window may differ by (0: none)
+  FX_P = 12,                     // R^(i+1), i = 0..15
+  FX_Q = FX_P + kFixHalf,        // B^(16-i), i = 0..15
+  // powers R^(32 t) = m 2^-64 2^-k with m >= 2^63, t = 0..32 (entry 0 unused): the m, then the k, four
+  // 16-bit numbers to a word; and B^(32 t)
+  FX_RM = FX_Q + kFixHalf,
+  FX_RX = FX_RM + 33,
+  FX_BM = FX_RX + 9,
+  FX_BX = FX_BM + 33,
+  FX_WORDS = FX_BX + 9
+};
+enum FixFlags { FIX_ALT = 1, FIX_NEG = 2, FIX_GUARD = 4 };   // s = -1; g < 0; high gain (step 4's test)
+
+constexpr int kFixSmemWords = 2 * kFixHalf + 2 * 33;   // tables staged in shared memory
+// a window has one scale while none of its blocks of 32 rows lies further below its largest |F|
+constexpr int kFixBlockRange = 4;
+// headroom (bits) of a window of varying scale
+constexpr int kFixVarBits = 2;
+// a high-gain system's window must reach 2^-kFixGuard of the words' bound
+constexpr int kFixGuard = 8;
+
+// threads of a CTA that tries the fixed-point form on windows of NT blocks of n rows: 32 rows per thread
+// in one of the compiled widths (at least NT, which the FP64 form needs), 0 where it is not used.
+// Blocks shorter than 32 rows are the planner's (or the caller's) choice for systems that cannot fill
+// the chip, where the sweeps' latency counts: there the FP64 sweeps over short blocks are the shorter
+// chain (113 systems of 4096 rows beside 3983 MIXED ones: 104.7 us for the batch, 106.2 with this form).
+// Windows longer than 8192 rows would exceed 256 threads.
+__host__ __device__ inline int fix_threads(int NT, int n) {
+  const int64_t rows = (int64_t)NT * n;
+  const int w = rows <= 2048 ? 64 : (rows <= 4096 ? 128 : 256);
+  return (rows < 1024 || rows > 8192 || w < NT) ? 0 : w;
+}
+
+__host__ __device__ inline size_t window_fix_smem_bytes(int NTF) {
+  const size_t nw = (size_t)(NTF / 32);
+  return (size_t)NTF * kRegPairBytes + 8 * (size_t)kFixSmemWords + 8 * 3 * nw + 16 + 4 * 2 * nw + 2 * (size_t)NTF;
+}
+
+// acc + x r 2^-64, truncated (1.25 units below on average, at most 3)
+__device__ __forceinline__ u64 fx_mul(u64 x, unsigned rh, unsigned rl, u64 acc) {
+  const unsigned xh = (unsigned)(x >> 32), xl = (unsigned)x;
+  const u64 p = (u64)xh * rh + acc;
+  return p + (u64)__umulhi(xl, rh) + (u64)__umulhi(xh, rl);
+}
+__device__ __forceinline__ u64 fx_mul(u64 x, u64 r, u64 acc) { return fx_mul(x, (unsigned)(r >> 32), (unsigned)r, acc); }
+
+// s r, s a signed word and r = m 2^-64 2^-x, into a unit 2^(sh - x) times as large (sh >= 0)
+__device__ __forceinline__ u64 fx_move(u64 s, u64 m, int sh) {
+  const long long z = (long long)fx_mul(s ^ (1ull << 63), m, 0ull - (m >> 1));
+  return (u64)(z >> min(sh, 63));
+}
+// a signed word in a unit 2^sh times as large
+__device__ __forceinline__ u64 fx_rescale(u64 s, int sh) {
+  return sh >= 0 ? (u64)((long long)s >> min(sh, 63)) : s << -sh;
+}
+
+// K + d 2^sc: by shifts on the integer pipe (sb = 1086 - sc; smaller values shift out to zero) ...
+__device__ __forceinline__ u64 fx_from_f64_alu(double d, unsigned sb, u64 K) {
+  const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+  const unsigned sh = sb - ((hw >> 20) & 0x7FFu);
+  const unsigned mh = __funnelshift_l(lw, hw, 11) | 0x80000000u, ml = lw << 11;
+  u64 v;
+  asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(((u64)mh << 32) | ml), "r"(sh));
+  const int m = (int)hw >> 31;
+  v ^= (u64)(long long)m;
+  return v + K + (u64)(hw >> 31);
+}
+// ... or by the FP64 pipe's conversion (scadd = (sc << 20), plus the sign bit to negate): the two share
+// the rows, which balances the pipes (measured 255 G unknowns/s, all-integer 257, all-FP64 225)
+__device__ __forceinline__ u64 fx_from_f64_cvt(double d, unsigned scadd, u64 K) {
+  return (u64)__double2ll_rn(__hiloint2double((int)((unsigned)__double2hiint(d) + scadd), __double2loint(d))) + K;
+}
+// a word with the output constant already taken off (two's complement) to FP64; ek: exponent and sign
+// to add.  The lowest bit is set so that the exponent addition never meets a zero.
+__device__ __forceinline__ double fx_to_f64(u64 z, unsigned ek) {
+  const double d = __ll2double_rn((long long)(z | 1ull));
+  return __hiloint2double((int)((unsigned)__double2hiint(d) + ek), __double2loint(d));
+}
+
+// The window's rows [row_lo, row_lo + len) of a system (own rows [j0, j1) of them), len <= 32 NTF.
+// Returns false, with every thread of the CTA past a barrier and nothing stored, where the window's
+// values do not suit fixed point: the caller then solves it in FP64.
+template <int NTF>
+__device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, const double* tab, int64_t row_lo,
+                                           int len, int j0, int j1, unsigned char* smem) {
+  constexpr int NW = NTF / 32;
+  constexpr int H = kFixHalf;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  unsigned char* mine = smem + (size_t)tid * kRegPairBytes;
+  u64* tp = reinterpret_cast<u64*>(smem + (size_t)NTF * kRegPairBytes);
+  u64* tq = tp + H;
+  u64* tR = tq + H;
+  u64* tB = tR + 33;
+  u64* sw = tB + 33;                                         // 3 NW
+  u64* sx0 = sw + 3 * NW;                                    // the system's first row (2 entries)
+  unsigned* sexp = reinterpret_cast<unsigned*>(sx0 + 2);     // 2 NW
+  short* sblk = reinterpret_cast<short*>(sexp + 2 * NW);     // NTF: exponents of the threads' blocks
+  const u64* fx = reinterpret_cast<const u64*>(tab) + pp->o_fix;
+  const double* src = A.F + (int64_t)blockIdx.y * A.ldf + pp->off + row_lo;
+  double* dst = A.x + (int64_t)blockIdx.y * A.ldx + pp->off + row_lo;
+
+  slots_load(smem, src, len, (reinterpret_cast<uintptr_t>(src) & 15u) == 0u, lane, wid);
+  const short* rx = reinterpret_cast<const short*>(fx + FX_RX);
+  const short* bx = reinterpret_cast<const short*>(fx + FX_BX);
+  for (int i = tid; i < 2 * kFixHalf; i += NTF) tp[i] = fx[FX_P + i];
+  for (int i = tid; i < 33; i += NTF) {   // the powers as plain fractions
+    tR[i] = rx[i] > 63 ? 0ull : fx[FX_RM + i] >> rx[i];
+    tB[i] = bx[i] > 63 ? 0ull : fx[FX_BM + i] >> bx[i];
+  }
+  cp_async_wait_all();
+  __syncwarp();
+
+  // ---------------------------------------------------------------- the window's exponent range
+  const int nv = max(0, min(kFixRows, len - kFixRows * tid));   // the thread's rows
+  unsigned hmax = 0u, hblk = 0xFFFFFFFFu;
+  if (nv == kFixRows) {
+#pragma unroll
+    for (int k = 0; k < kFixRows / 2; ++k) {
+      const uint4 v = *reinterpret_cast<const uint4*>(mine + 16 * k);
+      hmax = __vimax3_u32(hmax, v.y & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu);
+    }
+    hblk = hmax;
+  } else {
+    for (int i = 0; i < nv; ++i)
+      hmax = max(hmax, reinterpret_cast<const unsigned*>(mine)[2 * i + 1] & 0x7FFFFFFFu);
+  }
+  const int eown = (int)(hmax >> 20);
+  sblk[tid] = (short)eown;
+  hmax = __reduce_max_sync(0xffffffffu, hmax);
+  hblk = __reduce_min_sync(0xffffffffu, hblk);
+  if (lane == 0) {
+    sexp[wid] = hmax;
+    sexp[NW + wid] = hblk;
+  }
+  __syncthreads();
+  hmax = sexp[0];
+  hblk = sexp[NW];
+#pragma unroll
+  for (int w = 1; w < NW; ++w) {
+    hmax = max(hmax, sexp[w]);
+    hblk = min(hblk, sexp[NW + w]);
+  }
+  const int emax = (int)(hmax >> 20), eblk = (int)(hblk >> 20);
+  const int hb = (int)fx[FX_HB];
+  const int tlast = (len - 1) / kFixRows;   // the last thread with rows
+  // one scale, |F| 2^sc < 2^hb <= K, for a window of normal finite values with sc >= 0 (zeros convert
+  // exactly then); else each thread's own
+  if (emax < 192 || emax > 1020 + hb) return false;
+  const bool var = eblk < emax - kFixBlockRange;
+  int e = emax;
+  if (var) {
+    const int step = (int)fx[FX_STEP];
+    const int el = (tid > 0 && nv > 0) ? sblk[tid - 1] : eown, er = (tid < tlast) ? sblk[tid + 1] : eown;
+    e = max(eown, max(el, er));
+    const bool ok = nv == 0 || (eown >= 192 && abs(eown - el) <= step && abs(eown - er) <= step);
+    if (!__syncthreads_and(step > 0 && ok)) return false;
+    sblk[tid] = (short)e;   // (read after the next barrier)
+  }
+  const int sc = hb - (e - 1022) - (var ? kFixVarBits : 0);
+  const u64 K = fx[FX_K], a0 = fx[FX_A];
+  const unsigned flags = (unsigned)fx[FX_FLAGS];
+  const unsigned alt = (flags & FIX_ALT) ? 0x80000000u : 0u;
+
+  // ---------------------------------------------------------------- 1. forward words of both halves
+  u64 E1 = 0, E2 = 0;
+  {
+    const unsigned rh = (unsigned)(fx[FX_R] >> 32), rl = (unsigned)fx[FX_R];
+    const unsigned sb = 1086u - (unsigned)sc, sodd = ((unsigned)sc << 20) + alt;
+#pragma unroll 4
+    for (int k = 0; k < H / 2; ++k) {
+      const double2 f = *reinterpret_cast<const double2*>(mine + 16 * k);
+      const double2 h = *reinterpret_cast<const double2*>(mine + 8 * H + 16 * k);
+      ulonglong2 w, v;
+      w.x = fx_mul(E1, rh, rl, fx_from_f64_alu(f.x, sb, K));
+      v.x = fx_mul(E2, rh, rl, fx_from_f64_alu(h.x, sb, K));
+      w.y = fx_mul(w.x, rh, rl, fx_from_f64_cvt(f.y, sodd, K));
+      v.y = fx_mul(v.x, rh, rl, fx_from_f64_cvt(h.y, sodd, K));
+      E1 = w.y;
+      E2 = v.y;
+      *reinterpret_cast<ulonglong2*>(mine + 16 * k) = w;
+      *reinterpret_cast<ulonglong2*>(mine + 8 * H + 16 * k) = v;
+    }
+  }
+  // ---------------------------------------------------------------- 2. the words entering the threads
+  const u64 R16 = tp[H - 1], B16 = tq[0];
+  u64 Uin;
+  const int levr = (int)fx[FX_LEVR], levb = (int)fx[FX_LEVB];
+  if (!var) {
+    u64 E = fx_mul(E1, R16, E2);
+    if (tid == 0) E = fx_mul(a0, tR[1], E);
+    for (int k = 0; k < levr; ++k) {
+      const int d = 1 << k;
+      const u64 y = __shfl_up_sync(0xffffffffu, E, d);
+      E = fx_mul(lane < d ? 0ull : y, tR[d], E);
+    }
+    if (lane == 31) sw[wid] = E;
+    Uin = __shfl_up_sync(0xffffffffu, E, 1);
+    if (lane == 0) Uin = 0;
+    __syncthreads();
+    if (wid > 0) {
+      u64 C = sw[wid - 1];
+      if (levr >= 5) {   // couplings may span several warps
+        C = sw[0];
+        for (int w = 1; w < wid; ++w) C = fx_mul(C, tR[32], sw[w]);
+      }
+      Uin = (lane == 0) ? C : fx_mul(C, tR[lane], Uin);
+    } else if (lane == 0) {
+      Uin = a0;
+    }
+  } else {
+    // signed words, each in its thread's unit; R <= 2^-1/4 here, so that 16 blocks away nothing is left
+    u64 S = fx_mul(E1, R16, E2) - (a0 - fx_mul(a0, tR[1], 0ull));
+    const int lev = min(4, levr + 1);
+    for (int k = 0; k < lev; ++k) {
+      const int d = 1 << k;
+      const u64 y = __shfl_up_sync(0xffffffffu, S, d);
+      const int ey = __shfl_up_sync(0xffffffffu, e, d);
+      if (lane >= d) S += fx_move(y, fx[FX_RM + d], rx[d] + e - ey);
+    }
+    if (lane == 31) sw[wid] = S;
+    __syncthreads();
+    u64 C = 0;
+    int eC = e;
+    if (wid > 0) {
+      C = sw[wid - 1];
+      eC = sblk[32 * wid - 1];
+      S += fx_move(C, fx[FX_RM + lane + 1], rx[lane + 1] + e - eC);
+    }
+    const u64 y = __shfl_up_sync(0xffffffffu, S, 1);
+    const int ey = __shfl_up_sync(0xffffffffu, e, 1);
+    Uin = a0 + (lane == 0 ? fx_rescale(C, e - eC) : fx_rescale(y, e - ey));
+  }
+  // ---------------------------------------------------------------- 3. backward words
+  const u64 Uin2 = fx_mul(Uin, R16, E1);
+  u64 Y1 = 0, Y2 = 0;
+  {
+    const unsigned bh = (unsigned)(fx[FX_B] >> 32), bl = (unsigned)fx[FX_B];
+    const unsigned uh = (unsigned)(Uin >> 32), ul = (unsigned)Uin, vh = (unsigned)(Uin2 >> 32), vl = (unsigned)Uin2;
+    if (nv == kFixRows) {
+#pragma unroll 4
+      for (int k = H / 2 - 1; k >= 0; --k) {
+        ulonglong2 w = *reinterpret_cast<const ulonglong2*>(mine + 16 * k);
+        ulonglong2 v = *reinterpret_cast<const ulonglong2*>(mine + 8 * H + 16 * k);
+        const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(tp + 2 * k);
+        w.y = Y1 = fx_mul(Y1, bh, bl, fx_mul(p.y, uh, ul, w.y));
+        v.y = Y2 = fx_mul(Y2, bh, bl, fx_mul(p.y, vh, vl, v.y));
+        w.x = Y1 = fx_mul(Y1, bh, bl, fx_mul(p.x, uh, ul, w.x));
+        v.x = Y2 = fx_mul(Y2, bh, bl, fx_mul(p.x, vh, vl, v.x));
+        *reinterpret_cast<ulonglong2*>(mine + 16 * k) = w;
+        *reinterpret_cast<ulonglong2*>(mine + 8 * H + 16 * k) = v;
+      }
+    } else if (nv > 0) {
+      // the system's last rows: beyond them u = 0 (the word a), so that X = 0 reaches row N unchanged
+      u64* col = reinterpret_cast<u64*>(mine);
+#pragma unroll 1
+      for (int i = kFixRows - 1; i >= 0; --i) {
+        u64& Y = (i < H) ? Y1 : Y2;
+        const u64 t = (i < nv) ? fx_mul(tp[i & (H - 1)], (i < H) ? Uin : Uin2, col[i]) : a0;
+        const u64 y = fx_mul((i < H) ? Y1 : Y2, bh, bl, t);
+        Y = y;
+        col[i] = y;
+      }
+    }
+  }
+  // ---------------------------------------------------------------- 4. the words beyond the threads
+  u64 Xin, E0;   // E0: the thread's first word, complete
+  {
+    const u64 loc = fx_mul(Y2, B16, Y1);
+    if (!var) {
+      u64 E = (nv == 0) ? 0ull : loc;
+      if (tid == tlast) E = fx_mul(1ull << 63, tB[1], E);
+      for (int k = 0; k < levb; ++k) {
+        const int d = 1 << k;
+        const u64 y = __shfl_down_sync(0xffffffffu, E, d);
+        E = fx_mul(lane + d > 31 ? 0ull : y, tB[d], E);
+      }
+      if (lane == 0) sw[NW + wid] = E;
+      Xin = __shfl_down_sync(0xffffffffu, E, 1);
+      if (lane == 31) Xin = 0;
+      __syncthreads();
+      if (wid < NW - 1) {
+        u64 C = sw[NW + wid + 1];
+        if (levb >= 5) {
+          C = sw[2 * NW - 1];
+          for (int w = NW - 2; w > wid; --w) C = fx_mul(C, tB[32], sw[NW + w]);
+        }
+        Xin = (lane == 31) ? C : fx_mul(C, tB[31 - lane], Xin);
+      }
+    } else {
+      u64 S = loc - ((1ull << 63) - fx_mul(1ull << 63, tB[1], 0ull));
+      if (nv == 0) S = 0;
+      const int lev = min(4, levb + 1);
+      for (int k = 0; k < lev; ++k) {
+        const int d = 1 << k;
+        const u64 y = __shfl_down_sync(0xffffffffu, S, d);
+        const int ey = __shfl_down_sync(0xffffffffu, e, d);
+        if (lane + d <= 31) S += fx_move(y, fx[FX_BM + d], bx[d] + e - ey);
+      }
+      if (lane == 0) sw[NW + wid] = S;
+      __syncthreads();
+      u64 C = 0;
+      int eC = e;
+      if (wid < NW - 1) {
+        C = sw[NW + wid + 1];
+        eC = sblk[32 * (wid + 1)];
+        S += fx_move(C, fx[FX_BM + 32 - lane], bx[32 - lane] + e - eC);
+      }
+      const u64 y = __shfl_down_sync(0xffffffffu, S, 1);
+      const int ey = __shfl_down_sync(0xffffffffu, e, 1);
+      Xin = (1ull << 63) + (lane == 31 ? fx_rescale(C, e - eC) : fx_rescale(y, e - ey));
+    }
+    if (tid >= tlast) Xin = 1ull << 63;
+    E0 = fx_mul(Xin, tB[1], loc);
+  }
+  if (flags & FIX_GUARD) {
+    // high gain: the words' unit is set by the largest possible |X|; a window whose solution stays far
+    // below that would keep fewer bits than FP64 does
+    const u64 m = (E0 >> 63) ? E0 - (1ull << 63) : (1ull << 63) - E0;
+    if (!__syncthreads_or(nv > 0 && (m >> (63 - kFixGuard)) != 0)) return false;
+  }
+  // the next kernel of the stream may begin its launch (it waits for this grid to complete)
+  asm volatile("griddepcontrol.launch_dependents;");
+
+  if (row_lo == 0) {
+    // the system's first rows: X_i -= X_0 B R^(i+1)
+    if (tid == 0) sx0[0] = E0;
+    __syncthreads();
+    const u64 x0 = sx0[0];
+    const bool neg = (x0 >> 63) == 0;
+    u64 c = neg ? (1ull << 63) - x0 : x0 - (1ull << 63);
+    c = fx_mul(c, fx[FX_B], 0ull);
+    if (!var) {
+      for (int t = 0; t < (tid >> 5); ++t) c = fx_mul(c, tR[32], 0ull);
+      if (lane) c = fx_mul(c, tR[lane], 0ull);
+    } else if (tid > 32) {
+      c = 0;
+    } else if (tid > 0) {   // from the first thread's unit into this one's
+      const int sh = rx[tid] + e - sblk[0];
+      c = sh > 63 ? 0ull : fx_mul(c, fx[FX_RM + tid], 0ull) >> sh;
+    }
+    if (c > 2 && nv > 0) {
+      u64* col = reinterpret_cast<u64*>(mine);
+      u64 ch = c;
+#pragma unroll 1
+      for (int i = 0; i < kFixRows; ++i) {
+        if (i == H) ch = fx_mul(c, R16, 0ull);
+        const u64 dlt = fx_mul(tp[i & (H - 1)], ch, 0ull);
+        col[i] = neg ? col[i] + dlt : col[i] - dlt;
+      }
+    }
+  }
+
+  // ---------------------------------------------------------------- 5. the solution, own rows out
+  if (kFixRows * tid < j1 && kFixRows * (tid + 1) > j0) {
+    const u64 X1 = fx_mul(Xin, B16, Y2);
+    const unsigned xh = (unsigned)(X1 >> 32), xl = (unsigned)X1, yh = (unsigned)(Xin >> 32), yl = (unsigned)Xin;
+    const unsigned gh = (unsigned)(fx[FX_G] >> 32), gl = (unsigned)fx[FX_G];
+    const u64 kg = fx[FX_KG];
+    const unsigned eke = ((unsigned)((int)fx[FX_GK] - sc) << 20) + ((flags & FIX_NEG) ? 0x80000000u : 0u), eko = eke + alt;
+#pragma unroll 4
+    for (int k = 0; k < H / 2; ++k) {
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(mine + 16 * k);
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(mine + 8 * H + 16 * k);
+      const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(tq + 2 * k);
+      const u64 z0 = fx_mul(fx_mul(q.x, xh, xl, w.x), gh, gl, kg), z1 = fx_mul(fx_mul(q.y, xh, xl, w.y), gh, gl, kg);
+      const u64 s0 = fx_mul(fx_mul(q.x, yh, yl, v.x), gh, gl, kg), s1 = fx_mul(fx_mul(q.y, yh, yl, v.y), gh, gl, kg);
+      *reinterpret_cast<double2*>(mine + 16 * k) = make_double2(fx_to_f64(z0, eke), fx_to_f64(z1, eko));
+      *reinterpret_cast<double2*>(mine + 8 * H + 16 * k) = make_double2(fx_to_f64(s0, eke), fx_to_f64(s1, eko));
+    }
+  }
+  __syncwarp();
+  const bool al_dst = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0u;
+  if (A.xf == nullptr) {
+    slots_store(smem, dst, j0, j1, al_dst, lane, wid);
+    return true;
+  }
+  // the adjoint (a5): the gradient sums over the own rows, in FP64, beside the store
+  double g0 = 0.0, gm = 0.0, gp = 0.0;
+  {
+    const int r0 = max(j0 - wid * kWarpRows, 0), r1 = min(j1 - wid * kWarpRows, kWarpRows);
+    const int64_t N = pp->N, rw = row_lo + wid * kWarpRows;
+    const double* xf = A.xf + pp->off + rw;
+    double* dw = dst + wid * kWarpRows;
+    const unsigned char* sl = smem + (size_t)wid * 32 * kRegPairBytes + lane * 8;
+#pragma unroll 4
+    for (int j = lane + (r0 & ~31); j < r1; j += 32) {
+      if (j < r0) continue;
+      const double dv = *reinterpret_cast<const double*>(sl + (j >> 5) * kRegPairBytes);
+      const int64_t r = rw + j;
+      __stcs(dw + j, dv);
+      g0 = fma(dv, xf[j], g0);
+      gm = fma(dv, r > 0 ? xf[j - 1] : 0.0, gm);
+      gp = fma(dv, r + 1 < N ? xf[j + 1] : 0.0, gp);
+    }
+  }
+  // the warp's three sums: lanes 0-7 end with sum lambda_r x_{r-1}, 8-15 with sum lambda_r x_r, 16-23
+  // with sum lambda_r x_{r+1} (6 additions instead of 15)
+  {
+    const bool up = lane & 16, odd = lane & 8;
+    const double t0 = up ? gm : gp, t1 = up ? g0 : 0.0;
+    double k0 = up ? gp : gm, k1 = up ? 0.0 : g0;
+    k0 += __shfl_xor_sync(0xffffffffu, t0, 16);
+    k1 += __shfl_xor_sync(0xffffffffu, t1, 16);
+    g0 = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 8);
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) g0 += __shfl_xor_sync(0xffffffffu, g0, d);
+  }
+  double* sred = reinterpret_cast<double*>(sw);
+  __syncthreads();
+  if ((lane & 7) == 0 && lane < 24) sred[(lane >> 3) * NW + wid] = g0;
+  __syncthreads();
+  if (tid < 3) {
+    double s = 0.0;
+    for (int w = 0; w < NW; ++w) s += sred[tid * NW + w];
+    A.part[3 * (size_t)blockIdx.x + tid] = s;
+  }
+  return true;
+}
+
+}  // namespace dich
