@@ -178,7 +178,9 @@ int dichotomy_solve(dich_plan_t plan, const double* d_F, double* d_x, void* stre
  * right-hand sides F_k = d_F + k ldf, x_k = d_x + k ldx (k = 0 .. M-1; row-major [M][N] when
  * ldf = ldx = N).  The plan (the preliminary step) serves every right-hand side.  The single
  * and halo paths enqueue one kernel per 65535 right-hand sides; the general path three
- * kernels per right-hand side, in order on `stream`.  M = 1 is dichotomy_solve.
+ * kernels per right-hand side, in order on `stream`.  M = 1 is dichotomy_solve.  A series of
+ * enough right-hand sides to fill the GPU takes the default geometry where the plan's own was
+ * chosen for one (a short system's narrower windows): the same solutions up to rounding.
  * Errors: DICH_ERR_ARG (M < 0, ld < N for M > 1, null/misaligned/host pointers),
  * DICH_ERR_ALIAS (the F and x ranges overlap), DICH_ERR_UNBOUND, DICH_ERR_CUDA (launch). */
 int dichotomy_solve_series(dich_plan_t plan, int64_t M, const double* d_F, int64_t ldf, double* d_x,
