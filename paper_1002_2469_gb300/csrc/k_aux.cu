@@ -303,49 +303,51 @@ cudaError_t launch_block_scan_batched(const SysPlan* plans, const double* tabs, 
   return cudaGetLastError();
 }
 
+// One CTA per system.  Bound by latency (an FP64 addition is 64 clocks): one pass over the partial sums,
+// two barrier-free reductions in registers and one barrier, launched with programmatic stream
+// serialization like the window kernels.  (505 MIXED windows of one system: the whole adjoint takes
+// 15.2 us; with a plain launch and a shared-memory tree of eight barriers it took 17.3.)
 __global__ void __launch_bounds__(256) k_adj_finalize(const double* part, const int32_t* sys_ids,
                                                       const int64_t* first, const int64_t* count, int64_t count0,
                                                       double* gt) {
-  __shared__ double sh[3 * 256], she[3 * 256];
+  __shared__ double sh[3 * 8];
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the window kernel's sums are complete
+  asm volatile("griddepcontrol.launch_dependents;");
   const int64_t k = blockIdx.x;
   const int64_t s = sys_ids ? sys_ids[k] : k;
-  const int64_t f = first ? first[k] : 0;
   const int64_t c = count ? count[k] : count0;
-  // every addition's rounding error is kept (TwoSum) and added at the end: a few operations per CTA of
-  // the adjoint, and the sums are then as good as their per-CTA terms
-  double a[3] = {0.0, 0.0, 0.0}, e[3] = {0.0, 0.0, 0.0};
-  auto add = [](double& x, double& err, double y, double yerr) {
-    const double t = x + y, z = t - x;
-    err += ((x - (t - z)) + (y - z)) + yerr;
-    x = t;
-  };
-  for (int64_t i = threadIdx.x; i < c; i += 256)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) add(a[j], e[j], part[3 * (f + i) + j], 0.0);
-  for (int d = 128; d > 0; d >>= 1) {
-    const int at = (int)threadIdx.x;
-    if (at < 2 * d)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        sh[256 * j + at] = a[j];
-        she[256 * j + at] = e[j];
-      }
-    __syncthreads();
-    if (at < d)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) add(a[j], e[j], sh[256 * j + at + d], she[256 * j + at + d]);
-    __syncthreads();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const double* p = part + 3 * (first ? first[k] : 0);
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+  for (int64_t i = threadIdx.x; i < c; i += 256) {
+    a0 += p[3 * i];
+    a1 += p[3 * i + 1];
+    a2 += p[3 * i + 2];
   }
-  if (threadIdx.x == 0)
+  const double w = warp_sum3(a0, a1, a2, lane);
+  if ((lane & 7) == 0 && lane < 24) sh[8 * (lane >> 3) + wid] = w;
+  __syncthreads();
+  if (wid == 0) {
+    double v = lane < 24 ? sh[lane] : 0.0;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) gt[3 * s + j] = -(a[j] + e[j]);
+    for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if ((lane & 7) == 0 && lane < 24) gt[3 * s + (lane >> 3)] = -v;
+  }
 }
 
 cudaError_t launch_adj_finalize(const double* part, const int32_t* sys_ids, const int64_t* first,
                                 const int64_t* count, int64_t count0, int64_t nsys, double* gt, cudaStream_t st) {
   if (nsys <= 0) return cudaSuccess;
-  k_adj_finalize<<<(unsigned)nsys, 256, 0, st>>>(part, sys_ids, first, count, count0, gt);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nsys);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_adj_finalize, part, sys_ids, first, count, count0, gt);
 }
 
 // x = F / t_0 for one-row systems; adjoint form when w != nullptr:

@@ -65,6 +65,19 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // 2^k as a double for |k| <= 1000 (bit construction)
 __device__ __forceinline__ double pow2i(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
+// a warp's three sums: lanes 0-7 return the sum of x, 8-15 that of y, 16-23 that of z (6 additions
+// instead of the 15 of three shuffle trees)
+__device__ __forceinline__ double warp_sum3(double x, double y, double z, int lane) {
+  const bool up = lane & 16, odd = lane & 8;
+  double k0 = up ? z : x, k1 = up ? 0.0 : y;
+  k0 += __shfl_xor_sync(0xffffffffu, up ? x : z, 16);
+  k1 += __shfl_xor_sync(0xffffffffu, up ? y : 0.0, 16);
+  double v = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 8);
+#pragma unroll
+  for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+
 // barrier over the first NT threads of a CTA of NTF threads
 template <int NT, int NTF = NT>
 __device__ __forceinline__ void sync_first() {

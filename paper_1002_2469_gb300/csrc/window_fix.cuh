@@ -40,6 +40,7 @@
 // Layout: one 272-byte slot per thread (slots.cuh) (F, W, Y and x in turn, in place); loops
 // unrolled by two row pairs of both halves.
 #pragma once
+#include <type_traits>
 #include "slots.cuh"
 
 namespace dich {
@@ -292,31 +293,28 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
   {
     const unsigned bh = (unsigned)(fx[FX_B] >> 32), bl = (unsigned)fx[FX_B];
     const unsigned uh = (unsigned)(Uin >> 32), ul = (unsigned)Uin, vh = (unsigned)(Uin2 >> 32), vl = (unsigned)Uin2;
-    if (nv == kFixRows) {
+    // GUARD: the system's last rows lie in this thread; beyond them u = 0 (the word a), so that X = 0
+    // reaches row N unchanged
+    auto sweep = [&](auto guard_) {
+      constexpr bool GUARD = decltype(guard_)::value;
 #pragma unroll 4
       for (int k = H / 2 - 1; k >= 0; --k) {
         ulonglong2 w = *reinterpret_cast<const ulonglong2*>(mine + 16 * k);
         ulonglong2 v = *reinterpret_cast<const ulonglong2*>(mine + 8 * H + 16 * k);
         const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(tp + 2 * k);
-        w.y = Y1 = fx_mul(Y1, bh, bl, fx_mul(p.y, uh, ul, w.y));
-        v.y = Y2 = fx_mul(Y2, bh, bl, fx_mul(p.y, vh, vl, v.y));
-        w.x = Y1 = fx_mul(Y1, bh, bl, fx_mul(p.x, uh, ul, w.x));
-        v.x = Y2 = fx_mul(Y2, bh, bl, fx_mul(p.x, vh, vl, v.x));
+        auto u = [&](int i, u64 t) { return (GUARD && i >= nv) ? a0 : t; };
+        w.y = Y1 = fx_mul(Y1, bh, bl, u(2 * k + 1, fx_mul(p.y, uh, ul, w.y)));
+        v.y = Y2 = fx_mul(Y2, bh, bl, u(H + 2 * k + 1, fx_mul(p.y, vh, vl, v.y)));
+        w.x = Y1 = fx_mul(Y1, bh, bl, u(2 * k, fx_mul(p.x, uh, ul, w.x)));
+        v.x = Y2 = fx_mul(Y2, bh, bl, u(H + 2 * k, fx_mul(p.x, vh, vl, v.x)));
         *reinterpret_cast<ulonglong2*>(mine + 16 * k) = w;
         *reinterpret_cast<ulonglong2*>(mine + 8 * H + 16 * k) = v;
       }
-    } else if (nv > 0) {
-      // the system's last rows: beyond them u = 0 (the word a), so that X = 0 reaches row N unchanged
-      u64* col = reinterpret_cast<u64*>(mine);
-#pragma unroll 1
-      for (int i = kFixRows - 1; i >= 0; --i) {
-        u64& Y = (i < H) ? Y1 : Y2;
-        const u64 t = (i < nv) ? fx_mul(tp[i & (H - 1)], (i < H) ? Uin : Uin2, col[i]) : a0;
-        const u64 y = fx_mul((i < H) ? Y1 : Y2, bh, bl, t);
-        Y = y;
-        col[i] = y;
-      }
-    }
+    };
+    if (nv == kFixRows)
+      sweep(std::false_type());
+    else if (nv > 0)
+      sweep(std::true_type());
   }
   // ---------------------------------------------------------------- 4. the words beyond the threads
   u64 Xin, E0;   // E0: the thread's first word, complete
@@ -395,13 +393,20 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
       c = sh > 63 ? 0ull : fx_mul(c, fx[FX_RM + tid], 0ull) >> sh;
     }
     if (c > 2 && nv > 0) {
-      u64* col = reinterpret_cast<u64*>(mine);
-      u64 ch = c;
-#pragma unroll 1
-      for (int i = 0; i < kFixRows; ++i) {
-        if (i == H) ch = fx_mul(c, R16, 0ull);
-        const u64 dlt = fx_mul(tp[i & (H - 1)], ch, 0ull);
-        col[i] = neg ? col[i] + dlt : col[i] - dlt;
+      const u64 c2 = fx_mul(c, R16, 0ull);
+      const unsigned ch = (unsigned)(c >> 32), cl = (unsigned)c, dh = (unsigned)(c2 >> 32), dl = (unsigned)c2;
+      const u64 sg = neg ? 0ull : ~0ull;   // two's complement of the correction to subtract it
+#pragma unroll 4
+      for (int k = 0; k < H / 2; ++k) {
+        ulonglong2 w = *reinterpret_cast<const ulonglong2*>(mine + 16 * k);
+        ulonglong2 v = *reinterpret_cast<const ulonglong2*>(mine + 8 * H + 16 * k);
+        const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(tp + 2 * k);
+        w.x += (fx_mul(p.x, ch, cl, 0ull) ^ sg) - sg;
+        w.y += (fx_mul(p.y, ch, cl, 0ull) ^ sg) - sg;
+        v.x += (fx_mul(p.x, dh, dl, 0ull) ^ sg) - sg;
+        v.y += (fx_mul(p.y, dh, dl, 0ull) ^ sg) - sg;
+        *reinterpret_cast<ulonglong2*>(mine + 16 * k) = w;
+        *reinterpret_cast<ulonglong2*>(mine + 8 * H + 16 * k) = v;
       }
     }
   }
@@ -449,18 +454,7 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
       gp = fma(dv, r + 1 < N ? xf[j + 1] : 0.0, gp);
     }
   }
-  // the warp's three sums: lanes 0-7 end with sum lambda_r x_{r-1}, 8-15 with sum lambda_r x_r, 16-23
-  // with sum lambda_r x_{r+1} (6 additions instead of 15)
-  {
-    const bool up = lane & 16, odd = lane & 8;
-    const double t0 = up ? gm : gp, t1 = up ? g0 : 0.0;
-    double k0 = up ? gp : gm, k1 = up ? 0.0 : g0;
-    k0 += __shfl_xor_sync(0xffffffffu, t0, 16);
-    k1 += __shfl_xor_sync(0xffffffffu, t1, 16);
-    g0 = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 8);
-#pragma unroll
-    for (int d = 4; d > 0; d >>= 1) g0 += __shfl_xor_sync(0xffffffffu, g0, d);
-  }
+  g0 = warp_sum3(gm, g0, gp, lane);
   double* sred = reinterpret_cast<double*>(sw);
   __syncthreads();
   if ((lane & 7) == 0 && lane < 24) sred[(lane >> 3) * NW + wid] = g0;
