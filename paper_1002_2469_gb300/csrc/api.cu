@@ -788,10 +788,12 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
       delete p;
       return rc;
     }
-    // A multi-window system with fewer windows than twice the GPU's SMs is latency-bound: unless
+    // A system of some length with fewer windows than twice the GPU's SMs is latency-bound: unless
     // the caller fixed the geometry, take narrower windows, then shorter blocks, while the system
-    // stays on the halo path (halo at most half the window).  Measured on GB300: N = 65536 solves
-    // 2x faster with 64-thread windows of 2-row blocks than with the large-N default.
+    // is on the halo path (halo at most half the window).  Measured on GB300: N = 65536 solves
+    // 2x faster with 64-thread windows of 2-row blocks than with the large-N default; one window
+    // of FP64-form blocks of 10 rows and more is split the same way (N = 3001 with blocks of 47 rows 11.0 us, ten
+    // windows of 7-row blocks 6.8 us; N = 600, 10 rows: 8.1 and 6.1), shorter blocks gain nothing.
     // Coupling longer than half a default window, but not half a window of twice the width: with the
     // fixed-point form one pass over overlapping windows is the faster way (tridiag{-1, 2.001, -1},
     // N = 2^24 + 1: 120 us against 348 us for the general path's two FP64 passes; solved in FP64, where
@@ -819,7 +821,8 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
       }
     }
     const int sms = device_sms();
-    if (o.NT == 0 && o.n_req == 0 && p->path == PATH_HALO && p->tiles < 2 * (int64_t)sms) {
+    if (o.NT == 0 && o.n_req == 0 && (p->path == PATH_HALO || (p->path == PATH_SINGLE && p->form == FORM_F64 && n0 >= 10)) &&
+        p->tiles < 2 * (int64_t)sms) {
       const int nmin = (p->form == FORM_MIXED) ? 2 : 4;
       int NT = p->NT, n = n0;
       while (p->tiles < 2 * (int64_t)sms) {
