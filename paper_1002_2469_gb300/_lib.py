@@ -80,6 +80,8 @@ def lib_path() -> str:
 def load(build_if_missing: bool = True):
     """Load libdichotomy.so (building it with nvcc if it is missing or stale)."""
     global _lib_obj
+    if _lib_obj is not None:
+        return _lib_obj
     with _lock:
         if _lib_obj is not None:
             return _lib_obj

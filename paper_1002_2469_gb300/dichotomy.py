@@ -27,20 +27,28 @@ __all__ = [
 ]
 
 
-def _stream(stream) -> ctypes.c_void_p:
+# The raw handle of the current stream without a torch.cuda.Stream object around it (0.2 us a call
+# against 3.1 us of the 11 us that Plan.solve took on a Grace host).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        if _raw_stream is not None and _raw_device is not None:
+            return _raw_stream(_raw_device())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
-def _dev(t: torch.Tensor, name: str) -> ctypes.c_void_p:
+def _dev(t: torch.Tensor, name: str) -> int:
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor (the solver has no CPU path)")
     if t.dtype != torch.float64 or not t.is_contiguous():
         raise TypeError(f"{name} must be a contiguous float64 tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 # ------------------------------------------------------------------ C entry points
@@ -95,7 +103,7 @@ def _dev_rows(t: torch.Tensor, name: str):
         raise TypeError(f"{name} must be a CUDA tensor (the solver has no CPU path)")
     if t.dtype != torch.float64 or t.dim() != 2 or (t.shape[1] > 1 and t.stride(1) != 1):
         raise TypeError(f"{name} must be a 2-D float64 tensor with contiguous rows")
-    return ctypes.c_void_p(t.data_ptr()), int(t.stride(0))
+    return t.data_ptr(), int(t.stride(0))
 
 
 def dichotomy_solve_series(plan, F: torch.Tensor, x: torch.Tensor, stream=None) -> None:
