@@ -9,8 +9,8 @@ operator; mode k = 1..M leaves one tridiagonal Toeplitz system along y,
 
 the series of Sec. 3.2 with one t_0 per mode.  All M systems are solved as one batch by the
 Dichotomy kernels (the library's batched entry point); the inverse DST-I (the same transform)
-returns u.  The transforms use torch's FFT (cuFFT): DST-I of length M through a real FFT of
-length 2 (M + 1).
+returns u.  The transforms use torch's FFT (cuFFT) of length M + 1 with the library's kernels before
+and after it (two columns per complex row, transposed on the way in and out).
 
 Neumann conditions in y (bc_y="neumann"): My cell-centred unknowns y_j = (j + 1/2) / My with
 du/dy = 0 at y = 0 and y = 1 (ghost cells equal to their neighbours).  Mode k then leaves the
@@ -25,6 +25,7 @@ import math
 import numpy as np
 import torch
 
+from . import _lib
 from . import dichotomy as _d
 
 __all__ = ["dst1", "mode_t0", "Poisson2D"]
@@ -82,14 +83,32 @@ class Poisson2D:
         self.batch = _d.Batch(np.full(self.M, self.My, dtype=np.int64), -ones, t0, -ones, precision=precision,
                               **corners)
         self.device = device
+        # coefficients of the transforms' first step, for the right-hand side (with hy^2) and the modes
+        N = self.M + 1
+        s = np.sin(np.arange(N // 2 + 1) * (math.pi / N))
+        c = np.stack([s + 0.5, s - 0.5], axis=1) * (0.5 * math.sqrt(2.0 / N))
+        dev = self.batch.workspace.device
+        self._coef_f = torch.from_numpy(c * (self.hy * self.hy)).to(dev)
+        self._coef_v = torch.from_numpy(c).to(dev)
+
+    def _dst(self, a: torch.Tensor, coef: torch.Tensor) -> torch.Tensor:
+        """The orthonormal DST-I of a contiguous [M, My] array along its first axis, times the factor in coef."""
+        L, stream = _lib.load(), _d._stream(None)
+        z = torch.empty(((self.My + 1) // 2, self.M + 1), dtype=torch.complex128, device=a.device)
+        _lib.check(L.dichotomy_dst_pre(self.M, self.My, _d._dev(a, "f"), coef.data_ptr(), z.data_ptr(), stream),
+                   "dichotomy_dst_pre")
+        Z = torch.fft.fft(z, dim=-1)
+        out = torch.empty_like(a)
+        _lib.check(L.dichotomy_dst_post(self.M, self.My, Z.data_ptr(), out.data_ptr(), stream), "dichotomy_dst_post")
+        return out
 
     def solve(self, f: torch.Tensor) -> torch.Tensor:
         """u for the right-hand side f ([M, My], float64, CUDA)."""
         if f.shape != (self.M, self.My):
             raise ValueError(f"f must be [{self.M}, {self.My}]")
-        rhs = (self.hy * self.hy) * dst1(f, dim=0)                # [k, j]: mode k along y
+        rhs = self._dst(f.detach().contiguous(), self._coef_f)    # [k, j]: mode k along y
         v = self.batch.solve(rhs.reshape(-1)).reshape(self.M, self.My)
-        return dst1(v, dim=0)
+        return self._dst(v, self._coef_v)
 
     def status(self) -> int:
         return self.batch.status()

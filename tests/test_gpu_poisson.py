@@ -84,3 +84,21 @@ def test_poisson2d_neumann_y_manufactured(P):
     f = OP.laplacian5_neumann_y(us)
     u = P.Poisson2D(M, My=My, bc_y="neumann").solve(torch.from_numpy(f).cuda()).cpu().numpy()
     assert rel(u, us) < 1e-10
+
+
+@pytest.mark.parametrize("M,My", [(1, 1), (1, 5), (2, 3), (3, 64), (62, 65), (63, 63), (64, 129), (255, 17), (256, 16),
+                                  (257, 130), (511, 33), (1022, 31), (130, 1000)])
+def test_transform_steps_against_scipy(P, M, My):
+    """The transform of Poisson2D at the edges of its tiles (32 values of k and their mirror images by 64
+    columns; 128 values of m by 16 columns), odd and even lengths.  A DST of length M sums M products:
+    each output within (log2(M + 1) + 8) 2^-53 of the columns' 2-norm, the running sums of the odd
+    outputs within sqrt(M + 1) times that."""
+    import scipy.fft
+    a = np.random.default_rng(M + 7 * My).standard_normal((M, My))
+    solver = P.Poisson2D(M, My=My)
+    x = solver._dst(torch.from_numpy(a).cuda(), solver._coef_v).cpu().numpy()
+    ref = scipy.fft.dst(a, type=1, norm="ortho", axis=0)
+    tol = (math.log2(M + 1) + 8) * 2.0 ** -53 * np.linalg.norm(a, axis=0) * math.sqrt(M + 1)
+    assert np.all(np.abs(x - ref) <= tol)
+    scaled = solver._dst(torch.from_numpy(a).cuda(), solver._coef_f).cpu().numpy()
+    assert np.all(np.abs(scaled - solver.hy ** 2 * ref) <= 2 * solver.hy ** 2 * tol)
