@@ -86,9 +86,8 @@ enum {
                                         general matrices: any rows, judged by dich_plan_info.growth;
                                         check results with dichotomy_residual / dichotomy_gen_residual */
   /* MIXED-form window kernel of Toeplitz plans and batches (the results agree to rounding):
-   * the register path keeps a thread's two 16-row blocks in registers; the shared-memory path sweeps the window's tile in shared memory.
-   * Default: the register path for single plans, and for batches unless most of their
-   * MIXED windows are whole one-window systems (latency-bound windows, where occupancy wins). */
+   * the register path keeps a thread's two 16-row blocks in registers; the shared-memory path sweeps
+   * the window's tile in shared memory.  Default: the register path wherever its shape allows. */
   DICH_FLAG_REG_PATH = 32,           /* the register path wherever its window shape allows */
   DICH_FLAG_SMEM_PATH = 64           /* the shared-memory path for every window */
 };
