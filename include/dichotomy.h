@@ -341,6 +341,17 @@ void dichotomy_batch_destroy(dich_batch_t batch);
 int dichotomy_dst_pre(int64_t M, int64_t My, const double* d_a, const double* d_coef, double* d_z, void* stream);
 int dichotomy_dst_post(int64_t M, int64_t My, const double* d_Z, double* d_X, void* stream);
 
+/* The whole transform for N = M + 1 = 512, 1024, 2048 or 4096, in 64-bit fixed point on the integer
+ * pipes (each column in its own power-of-two unit; results as close to the exact transform as an FP64
+ * FFT's): d_X = 2 scale sum_j d_a[j] sin(pi j k / N).  d_table: N pairs of 64-bit words
+ * ((cos t + 1) / 2, (1 - sin t) / 2) 2^64, t = 2 pi m / N, then N / 2 + 1 words sin(pi k / N) 2^64, all
+ * rounded and at most 2^64 - 1; d_work: 2 ceil(My / 2) N doubles; both 16-byte aligned.  d_X may be d_a.
+ * Enqueues three kernels (and clears one row of d_work for an odd My).
+ * Errors: DICH_ERR_ARG (another M, null, misaligned or host pointers), DICH_ERR_UNSUPPORTED (sizes past
+ * 2^31 tiles), DICH_ERR_CUDA. */
+int dichotomy_dst(int64_t M, int64_t My, const double* d_a, const void* d_table, double scale, double* d_work,
+                  double* d_X, void* stream);
+
 /* ---------------------------------------------------------------- misc */
 const char* dichotomy_strerror(int status);
 /* The last CUDA error string seen by this thread (empty if none). */

@@ -15,7 +15,8 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libdichotomy.so")
 SOURCES = ["api.cu", "k_f64.cu", "k_f64_64.cu", "k_f64_128.cu", "k_f64_256.cu", "k_mixed.cu", "k_mixed_64.cu",
-           "k_mixed_128.cu", "k_mixed_256.cu", "k_aux.cu", "noalloc.cu", "general.cu", "dst.cu"]
+           "k_mixed_128.cu", "k_mixed_256.cu", "k_aux.cu", "noalloc.cu", "general.cu", "dst.cu",
+           "dst_fixed.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

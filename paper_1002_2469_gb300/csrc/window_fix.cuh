@@ -41,11 +41,10 @@
 // unrolled by two row pairs of both halves.
 #pragma once
 #include <type_traits>
+#include "fixed.cuh"
 #include "slots.cuh"
 
 namespace dich {
-
-typedef unsigned long long u64;
 
 constexpr int kFixRows = 32;     // rows per thread
 constexpr int kFixHalf = 16;
@@ -93,14 +92,6 @@ __host__ __device__ inline size_t window_fix_smem_bytes(int NTF) {
   return (size_t)NTF * kRegPairBytes + 8 * (size_t)kFixSmemWords + 8 * 3 * nw + 16 + 4 * 2 * nw + 2 * (size_t)NTF;
 }
 
-// acc + x r 2^-64, truncated (1.25 units below on average, at most 3)
-__device__ __forceinline__ u64 fx_mul(u64 x, unsigned rh, unsigned rl, u64 acc) {
-  const unsigned xh = (unsigned)(x >> 32), xl = (unsigned)x;
-  const u64 p = (u64)xh * rh + acc;
-  return p + (u64)__umulhi(xl, rh) + (u64)__umulhi(xh, rl);
-}
-__device__ __forceinline__ u64 fx_mul(u64 x, u64 r, u64 acc) { return fx_mul(x, (unsigned)(r >> 32), (unsigned)r, acc); }
-
 // s r, s a signed word and r = m 2^-64 2^-x, into a unit 2^(sh - x) times as large (sh >= 0)
 __device__ __forceinline__ u64 fx_move(u64 s, u64 m, int sh) {
   const long long z = (long long)fx_mul(s ^ (1ull << 63), m, 0ull - (m >> 1));
@@ -111,17 +102,7 @@ __device__ __forceinline__ u64 fx_rescale(u64 s, int sh) {
   return sh >= 0 ? (u64)((long long)s >> min(sh, 63)) : s << -sh;
 }
 
-// K + d 2^sc: by shifts on the integer pipe (sb = 1086 - sc; smaller values shift out to zero) ...
-__device__ __forceinline__ u64 fx_from_f64_alu(double d, unsigned sb, u64 K) {
-  const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
-  const unsigned sh = sb - ((hw >> 20) & 0x7FFu);
-  const unsigned mh = __funnelshift_l(lw, hw, 11) | 0x80000000u, ml = lw << 11;
-  u64 v;
-  asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(((u64)mh << 32) | ml), "r"(sh));
-  const int m = (int)hw >> 31;
-  v ^= (u64)(long long)m;
-  return v + K + (u64)(hw >> 31);
-}
+// K + d 2^sc by shifts (fx_from_f64_alu, fixed.cuh) ...
 // ... or by the FP64 pipe's conversion (scadd = (sc << 20), plus the sign bit to negate): the two share
 // the rows, which balances the pipes (measured 255 G unknowns/s, all-integer 257, all-FP64 225)
 __device__ __forceinline__ u64 fx_from_f64_cvt(double d, unsigned scadd, u64 K) {

@@ -9,8 +9,9 @@ operator; mode k = 1..M leaves one tridiagonal Toeplitz system along y,
 
 the series of Sec. 3.2 with one t_0 per mode.  All M systems are solved as one batch by the
 Dichotomy kernels (the library's batched entry point); the inverse DST-I (the same transform)
-returns u.  The transforms use torch's FFT (cuFFT) of length M + 1 with the library's kernels before
-and after it (two columns per complex row, transposed on the way in and out).
+returns u.  Transforms of length M + 1 = 512 to 4096, a power of two, are the library's own (64-bit fixed
+point on the integer pipes); the others use torch's FFT (cuFFT) of length M + 1 with the library's
+kernels before and after it (two columns per complex row, transposed on the way in and out).
 
 Neumann conditions in y (bc_y="neumann"): My cell-centred unknowns y_j = (j + 1/2) / My with
 du/dy = 0 at y = 0 and y = 1 (ghost cells equal to their neighbours).  Mode k then leaves the
@@ -29,6 +30,9 @@ from . import _lib
 from . import dichotomy as _d
 
 __all__ = ["dst1", "mode_t0", "Poisson2D"]
+
+# transform lengths M + 1 with the library's own fixed-point FFT; others go through torch's FFT
+_FIXED = (512, 1024, 2048, 4096)
 
 
 def dst1(a: torch.Tensor, dim: int = 0) -> torch.Tensor:
@@ -61,6 +65,24 @@ def mode_t0(M: int) -> np.ndarray:
     return 2.0 + 4.0 * np.sin(k * math.pi / (2.0 * (M + 1))) ** 2
 
 
+def _transform_table(N: int) -> np.ndarray:
+    """The table of dichotomy_dst: N twiddles and N / 2 + 1 sines as 64-bit fractions (from extended
+    precision, at least 64 bits on both x86 and AArch64 hosts)."""
+    pi = np.longdouble("3.14159265358979323846264338327950288")
+    quarter = np.sin(np.arange(N // 4 + 1, dtype=np.longdouble) * (2 * pi / N))     # sin 2 pi m / N, a quarter
+    m = np.arange(N)
+    r = m % (N // 2)
+    sin = np.where(m < N // 2, 1, -1) * quarter[np.minimum(r, N // 2 - r)]
+    cos = sin[(m + N // 4) % N]
+    sine = np.sin(np.arange(N // 2 + 1, dtype=np.longdouble) * (pi / N))
+    w = np.concatenate([np.stack([(cos + 1) / 2, (1 - sin) / 2], axis=1).ravel(), sine])
+    one = w >= 1
+    words = np.where(one, np.longdouble(0), w * np.longdouble(2.0 ** 64)).astype(np.uint64)
+    words[one] = np.uint64(0xFFFFFFFFFFFFFFFF)
+    words[:2 * N] &= np.uint64(0xFFFFFFFFFFFFFFFE)                                   # twiddle words are even
+    return words
+
+
 class Poisson2D:
     """Solver for an [M, My] grid (My = M by default): Dirichlet in x; Dirichlet (My interior
     nodes, hy = 1 / (My + 1)) or Neumann (My cell centres, hy = 1 / My) in y.  The batch of M
@@ -86,14 +108,28 @@ class Poisson2D:
         # coefficients of the transforms' first step, for the right-hand side (with hy^2) and the modes
         N = self.M + 1
         s = np.sin(np.arange(N // 2 + 1) * (math.pi / N))
+        self._table = None
+        if N in _FIXED:
+            words = _transform_table(N)
+            dev = self.batch.workspace.device
+            self._table = torch.from_numpy(words.view(np.int64)).to(dev)
+            self._scale = 0.5 * math.sqrt(2.0 / N)
+            return
         c = np.stack([s + 0.5, s - 0.5], axis=1) * (0.5 * math.sqrt(2.0 / N))
         dev = self.batch.workspace.device
         self._coef_f = torch.from_numpy(c * (self.hy * self.hy)).to(dev)
         self._coef_v = torch.from_numpy(c).to(dev)
 
-    def _dst(self, a: torch.Tensor, coef: torch.Tensor) -> torch.Tensor:
-        """The orthonormal DST-I of a contiguous [M, My] array along its first axis, times the factor in coef."""
+    def _dst(self, a: torch.Tensor, factor: float) -> torch.Tensor:
+        """The orthonormal DST-I of a contiguous [M, My] array along its first axis, times factor (1 or hy^2)."""
         L, stream = _lib.load(), _d._stream(None)
+        if self._table is not None:
+            out = torch.empty_like(a)
+            work = torch.empty((self.My + 1) // 2 * 2 * (self.M + 1), dtype=torch.float64, device=a.device)
+            _lib.check(L.dichotomy_dst(self.M, self.My, _d._dev(a, "f"), self._table.data_ptr(), self._scale * factor,
+                                       work.data_ptr(), out.data_ptr(), stream), "dichotomy_dst")
+            return out
+        coef = self._coef_v if factor == 1.0 else self._coef_f
         z = torch.empty(((self.My + 1) // 2, self.M + 1), dtype=torch.complex128, device=a.device)
         _lib.check(L.dichotomy_dst_pre(self.M, self.My, _d._dev(a, "f"), coef.data_ptr(), z.data_ptr(), stream),
                    "dichotomy_dst_pre")
@@ -106,9 +142,9 @@ class Poisson2D:
         """u for the right-hand side f ([M, My], float64, CUDA)."""
         if f.shape != (self.M, self.My):
             raise ValueError(f"f must be [{self.M}, {self.My}]")
-        rhs = self._dst(f.detach().contiguous(), self._coef_f)    # [k, j]: mode k along y
+        rhs = self._dst(f.detach().contiguous(), self.hy * self.hy)    # [k, j]: mode k along y
         v = self.batch.solve(rhs.reshape(-1)).reshape(self.M, self.My)
-        return self._dst(v, self._coef_v)
+        return self._dst(v, 1.0)
 
     def status(self) -> int:
         return self.batch.status()

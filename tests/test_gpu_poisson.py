@@ -87,7 +87,8 @@ def test_poisson2d_neumann_y_manufactured(P):
 
 
 @pytest.mark.parametrize("M,My", [(1, 1), (1, 5), (2, 3), (3, 64), (62, 65), (63, 63), (64, 129), (255, 17), (256, 16),
-                                  (257, 130), (511, 33), (1022, 31), (130, 1000)])
+                                  (257, 130), (511, 33), (1022, 31), (130, 1000), (511, 1), (1023, 64), (2047, 35),
+                                  (4095, 66)])
 def test_transform_steps_against_scipy(P, M, My):
     """The transform of Poisson2D at the edges of its tiles (32 values of k and their mirror images by 64
     columns; 128 values of m by 16 columns), odd and even lengths.  A DST of length M sums M products:
@@ -96,9 +97,37 @@ def test_transform_steps_against_scipy(P, M, My):
     import scipy.fft
     a = np.random.default_rng(M + 7 * My).standard_normal((M, My))
     solver = P.Poisson2D(M, My=My)
-    x = solver._dst(torch.from_numpy(a).cuda(), solver._coef_v).cpu().numpy()
+    x = solver._dst(torch.from_numpy(a).cuda(), 1.0).cpu().numpy()
     ref = scipy.fft.dst(a, type=1, norm="ortho", axis=0)
     tol = (math.log2(M + 1) + 8) * 2.0 ** -53 * np.linalg.norm(a, axis=0) * math.sqrt(M + 1)
     assert np.all(np.abs(x - ref) <= tol)
-    scaled = solver._dst(torch.from_numpy(a).cuda(), solver._coef_f).cpu().numpy()
+    scaled = solver._dst(torch.from_numpy(a).cuda(), solver.hy ** 2).cpu().numpy()
     assert np.all(np.abs(scaled - solver.hy ** 2 * ref) <= 2 * solver.hy ** 2 * tol)
+
+
+@pytest.mark.parametrize("M", [511, 1023, 2047, 4095])
+def test_fixed_point_transform_of_uneven_columns(P, M):
+    """Columns of very different magnitudes in one pair (each has its own unit), zero columns, single
+    spikes, constants and alternating signs (the largest growth a pass can see), the ends of the FP64
+    range.  Per column: two units (below 2^-55 of the largest |a| times the growth sqrt(M) of its 2-norm)
+    per pass, product and running sum stay within (log2(M + 1) + 8) 2^-53 of its 2-norm times sqrt(M + 1),
+    as for the FP64 transform."""
+    import scipy.fft
+    rng = np.random.default_rng(M)
+    cols = [rng.standard_normal(M) * 1e-280, rng.standard_normal(M) * 1e280, np.zeros(M), np.ones(M),
+            (-1.0) ** np.arange(M), np.eye(M)[M // 2], np.eye(M)[0] * 5e-300, rng.standard_normal(M),
+            np.sin(np.arange(1, M + 1) * (math.pi / (M + 1))), 1e12 + rng.standard_normal(M),
+            np.exp(-0.05 * np.arange(M))]
+    a = np.stack(cols, axis=1)
+    solver = P.Poisson2D(M, My=a.shape[1])
+    x = solver._dst(torch.from_numpy(a).cuda(), 1.0).cpu().numpy()
+    unit = np.max(np.abs(a), axis=0)
+    unit[unit == 0.0] = 1.0
+    ref = scipy.fft.dst(a / unit, type=1, norm="ortho", axis=0)
+    tol = (math.log2(M + 1) + 8) * 2.0 ** -53 * np.linalg.norm(a / unit, axis=0) * math.sqrt(M + 1)
+    assert np.all(np.abs(x / unit - ref) <= tol)
+    bad = a.copy()
+    bad[3, 7] = np.nan
+    y = solver._dst(torch.from_numpy(bad).cuda(), 1.0).cpu().numpy()
+    assert np.isnan(y[:, 7]).all()   # and the pair's other column stands
+    assert np.all(np.abs(y[:, 6] / unit[6] - ref[:, 6]) <= tol[6])
