@@ -1429,7 +1429,7 @@ struct dich_batch_s {
   }
   int64_t nsys = 0;
   Opts opts;
-  bool reg_path = true;                   // MIXED windows on the register path (else shared memory)
+  int reg_path = 1;                       // MIXED windows on the register path (WinArgs::reg_path)
   // a second stream for the FP64-form windows when a batch has both forms: the two launches
   // overlap (fork/join through events on the caller's stream; CUDA-graph capture follows them)
   cudaStream_t aux = nullptr;
@@ -1592,7 +1592,13 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
   if (b->ntf) b->ntf = fix_threads(b->NT[FORM_F64], b->n_smem[FORM_F64]);
   // MIXED windows take the register path wherever its shape allows (one-window systems too: 3946 Poisson
   // modes of 4096 rows 80.9 us, on the shared-memory path 93.0)
-  b->reg_path = (o.flags & DICH_FLAG_SMEM_PATH) == 0;
+  // -- in the kernel that also takes shorter last blocks where at least an eighth of the windows have one
+  {
+    int64_t rag = 0;
+    for (int64_t s : order)
+      if (b->form[s] == FORM_MIXED && b->fwd[s].rec.n == kRegRows && b->fwd[s].rec.nlast < kRegRows) ++rag;
+    b->reg_path = (o.flags & DICH_FLAG_SMEM_PATH) ? 0 : (8 * rag >= (int64_t)b->items[FORM_MIXED].size() && rag > 0) ? 2 : 1;
+  }
   // general-path systems: block offsets in the shared buffers, windows without halo, scan chunks
   for (int32_t s : b->general) {
     SysPlan& rf = b->fwd[(size_t)s].rec;
@@ -1834,7 +1840,7 @@ static int batch_launch(dich_batch_t b, const double* F, double* x, const double
     a.check_finite = (b->opts.flags & DICH_FLAG_CHECK_FINITE) ? 1 : 0;
     a.n_smem = b->n_smem[f];
     a.sys_offset = sys_offset;
-    a.reg_path = b->reg_path ? 1 : 0;   // batch vectors are device memory
+    a.reg_path = b->reg_path;   // batch vectors are device memory
     const size_t smem = smem_bytes(b->NT[f], a.n_smem, f, b->ntf);
     cudaError_t e = (f == FORM_F64) ? launch_window_f64(b->NT[f], b->ntf, (int)nitems, smem, sf, a)
                                     : launch_window_mixed(b->NT[f], (int)nitems, smem, sf, a);

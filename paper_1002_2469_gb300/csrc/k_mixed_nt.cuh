@@ -7,7 +7,7 @@
 namespace dich {
 
 // KIND: the adjoint's instantiations (gradient sums in the store loop) when a.xf is set, else the
-// forward ones; the register-path kind when a.reg_path is set, else the shared-memory one
+// forward ones; the register-path kinds when a.reg_path is set, else the shared-memory one
 // (six CTAs per SM)
 template <int NT, int KIND>
 static cudaError_t launch_one(int grid, int grid_y, size_t smem, cudaStream_t st, const WinArgs& a) {
@@ -33,6 +33,7 @@ template <int NT>
 static cudaError_t launch_kind(int grid, int grid_y, size_t smem, cudaStream_t st, const WinArgs& a) {
   if (a.xf != nullptr)
     return a.reg_path ? launch_one<NT, KIND_REGADJ>(grid, grid_y, smem, st, a) : launch_one<NT, KIND_ADJ>(grid, grid_y, smem, st, a);
+  if (a.reg_path == 2) return launch_one<NT, KIND_REGRAG>(grid, grid_y, smem, st, a);
   if (a.reg_path) return launch_one<NT, KIND_REG>(grid, grid_y, smem, st, a);
   return launch_one<NT, KIND_SMEM>(grid, grid_y, smem, st, a);
 }

@@ -48,6 +48,7 @@ struct WinArgs {
   int64_t ldf, ldx;       // series: right-hand side blockIdx.y starts at F + y ldf, its solution at x + y ldx
   int64_t win0;           // single system: window of CTA blockIdx.x is win0 + blockIdx.x
   int32_t reg_path;       // F and x are device memory: windows of the register path's shape may take it
+                          // (2: also those with a shorter last block)
 };
 
 // shared memory bytes for a window kernel of width NT and n_smem rows

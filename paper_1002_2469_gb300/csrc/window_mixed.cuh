@@ -310,7 +310,10 @@ __host__ __device__ inline size_t window2_smem_bytes(int NT, int n_smem) {
 // KIND_ADJ -- the adjoint (shared-memory path, gradient sums in the store loop, six CTAs per SM).
 // KIND_REGADJ -- the adjoint with the register path for the windows it serves (up to 128 registers:
 // four CTAs per SM; its slots hold x during the tree).
-enum WinKind : int { KIND_REG = 0, KIND_ADJ = 1, KIND_SMEM = 2, KIND_REGADJ = 3 };
+// KIND_REGRAG -- KIND_REG with the register path also for windows whose last block is shorter, for launches
+// where many windows are of that kind (4000 systems of 4095 rows: 96 us against 147); where few are, the
+// larger kernel costs more than they gain (2^26 rows 231 -> 240 us, 1500 uneven systems 830 -> 864).
+enum WinKind : int { KIND_REG = 0, KIND_ADJ = 1, KIND_SMEM = 2, KIND_REGADJ = 3, KIND_REGRAG = 4 };
 
 template <int NT, int KIND>
 __global__ void __launch_bounds__(NT, (KIND == KIND_REGADJ ? 512 : 768) / NT)
@@ -369,10 +372,11 @@ __global__ void __launch_bounds__(NT, (KIND == KIND_REGADJ ? 512 : 768) / NT)
   const int64_t row_lo = wlo * (int64_t)n;
   const int len = nwin * n - (has_last ? (n - nlast) : 0);
 
-  if constexpr (KIND == KIND_REG || KIND == KIND_REGADJ) {
-    // 16-row blocks, all of full size: the register path
-    if (A.reg_path && A.mode == MODE_FULL && n == kRegRows && (!has_last || nlast == kRegRows) && !A.check_finite) {
-      window_reg<NT, ADJ>(A, pp, tab, P, wlo, nwin, hl, nown, row_lo, reinterpret_cast<unsigned char*>(sm));
+  if constexpr (KIND == KIND_REG || KIND == KIND_REGADJ || KIND == KIND_REGRAG) {
+    // 16-row blocks (KIND_REGRAG: the last one may be shorter): the register path
+    constexpr bool RAGK = KIND == KIND_REGRAG;
+    if (A.reg_path && A.mode == MODE_FULL && n == kRegRows && (RAGK || !has_last || nlast == kRegRows) && !A.check_finite) {
+      window_reg<NT, ADJ, RAGK>(A, pp, tab, P, wlo, nwin, hl, nown, row_lo, len, reinterpret_cast<unsigned char*>(sm));
       return;
     }
   }

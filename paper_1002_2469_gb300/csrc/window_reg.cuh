@@ -1,8 +1,8 @@
 // window_reg.cuh -- the register-resident path of the MIXED window kernel (16-row blocks).
 //
-// A window whose blocks all have 16 rows, whose right-hand side and solution are 16-byte aligned
-// device memory and whose launch asks for the full solve (MODE_FULL, forward) is solved with a
-// thread's pair of blocks (2 x 16 unknowns) kept in registers from the load to the store:
+// A window of 16-row blocks (forward: the system's last block may be shorter) whose launch asks for the
+// full solve (MODE_FULL) is solved with a thread's pair of blocks (2 x 16 unknowns) kept in registers
+// from the load to the store:
 //   - the window's rows of F arrive by 16-byte cp.async copies (8-byte ones where F is not 16-byte
 //     aligned), consecutive threads copying consecutive elements, into shared-memory slots of 272
 //     bytes, one per thread (its two blocks, 256 contiguous bytes, plus 16 bytes of padding, so that
@@ -33,12 +33,13 @@ struct Recs2;
 // block-coefficient record, the four beta coefficients and the 66 pair-map powers
 constexpr int kMidRec = 0, kMidK = 10, kMidPow = 14, kMidEntries = 80;
 
-// shared memory of the register path for NT threads: the pair slots, the two spike tables, the
+// shared memory of the register path for NT threads: the pair slots, the two spike tables (and those of
+// the thread that holds a shorter last block), the
 // warp-boundary first/last values, the scan scratch, the exponent maxima (of the right-hand side
 // and, for the adjoint, of the forward solution) and the middle record's entries
 __host__ __device__ inline size_t window_reg_smem_bytes(int NT) {
   const size_t nw = (size_t)(NT / 32);
-  return (size_t)NT * kRegPairBytes + 2 * 16 * (size_t)kRegRows + 8 * 2 * nw + 8 * 4 * nw + 4 * 4 * nw +
+  return (size_t)NT * kRegPairBytes + 4 * 16 * (size_t)kRegRows + 8 * 2 * nw + 8 * 4 * nw + 4 * 4 * nw +
          8 * (size_t)kMidEntries;
 }
 
@@ -158,9 +159,9 @@ __device__ __forceinline__ void tree_mid(const float2* tf, int rm, int pw, const
 // rows go to A.part (three per CTA).  The forward solution x (A.xf) comes into the pair slots by a
 // second copy as soon as w has moved to registers, and is read back row by row as lambda is
 // written over it.
-template <int NT, bool ADJ = false>
+template <int NT, bool ADJ, bool RAGK>
 __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, const double* tab, int64_t P,
-                                           int64_t wlo, int nwin, int hl, int nown, int64_t row_lo,
+                                           int64_t wlo, int nwin, int hl, int nown, int64_t row_lo, int len,
                                            unsigned char* smem) {
   constexpr int NW = NT / 32;
   constexpr int R = kRegRows;
@@ -168,7 +169,9 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
   unsigned char* mine = smem + (size_t)tid * kRegPairBytes;
   float4* tv4 = reinterpret_cast<float4*>(smem + (size_t)NT * kRegPairBytes);   // spikes, both lanes
   float4* tw4 = tv4 + R;
-  ffv* sbd = reinterpret_cast<ffv*>(tw4 + R);                                   // 2 NW warp-boundary values
+  float4* rv4 = tw4 + R;                                                         // the shorter last block's thread
+  float4* rw4 = rv4 + R;
+  ffv* sbd = reinterpret_cast<ffv*>(rw4 + R);                                   // 2 NW warp-boundary values
   ffv* swv = sbd + 2 * NW;                                                       // 4 NW scan scratch
   unsigned* sexp = reinterpret_cast<unsigned*>(swv + 4 * NW);                    // 2 NW exponent maxima
   unsigned* sexpx = sexp + 2 * NW;                                               // the same for x
@@ -183,7 +186,7 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
 
   const bool al_src = (reinterpret_cast<uintptr_t>(src) & 15u) == 0u, al_dst = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0u;
   // ---------------------------------------------------------------- F -> the pair slots (async)
-  slots_load(smem, src, nwin * R, al_src, lane, wid);
+  slots_load(smem, src, len, al_src, lane, wid);
   if constexpr (!ADJ) {   // (the adjoint, at four CTAs per SM, reads them from the tables: measured faster)
     const float2* tf = reinterpret_cast<const float2*>(tab);
     for (int i = tid; i < kMidEntries; i += NT) {
@@ -198,8 +201,29 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     tv4[tid] = make_float4(v.x, v.x, v.y, v.y);
     tw4[tid] = make_float4(w.x, w.x, w.y, w.y);
   }
+  // RAGK: a last block of fewer rows (forward only): its thread takes spike tables of its own, the last block's
+  // spikes in that block's lane (zero past its rows) beside the full blocks' in the other
+  const bool rag = RAGK && len < nwin * R;
+  const int nl = R - (nwin * R - len);                 // the last block's rows
+  const bool ragt = rag && (last0 || last1);           // this thread holds it
+  if (rag && tid < R) {
+    const float2* tf = reinterpret_cast<const float2*>(tab);
+    const bool lastx = (nwin & 1) != 0;                // its lane
+    const float2 v = (tid < pp->Lv) ? tf[pp->o_vf + tid] : make_float2(0.f, 0.f);
+    const float2 w = (tid < pp->Lw) ? tf[pp->o_wf + tid] : make_float2(0.f, 0.f);
+    // row R - 1 - tid of the block (rw4's index): nl - 1 - row from its end
+    const float2 vl = (tid < nl) ? tf[pp->o_vlf + tid] : make_float2(0.f, 0.f);
+    const int back = nl - 1 - (R - 1 - tid);
+    const float2 wl = (back >= 0) ? tf[pp->o_wlf + back] : make_float2(0.f, 0.f);
+    rv4[tid] = lastx ? make_float4(vl.x, v.x, vl.y, v.y) : make_float4(v.x, vl.x, v.y, vl.y);
+    rw4[tid] = lastx ? make_float4(wl.x, w.x, wl.y, w.y) : make_float4(w.x, wl.x, w.y, wl.y);
+  }
   cp_async_wait_all();
   __syncwarp();   // (the tables staged above are read after the exponent range's barrier)
+  if (rag && ragt) {   // rows past the system's end: a value of the block (for the exponent range), zeroed below
+    double* col = reinterpret_cast<double*>(mine + (last1 ? 8 * R : 0));
+    for (int i = nl; i < R; ++i) col[i] = col[0];
+  }
 
   // ---------------------------------------------------------------- the pair in registers
   // a[k] = rows 2k, 2k+1 of block 2t; b[k] the same of block 2t+1.  The slot part of an inactive
@@ -263,7 +287,8 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
   const int ghw = __double2hiint(pp->g);
   const bool gfold = ((ghw >> 20) & 0x7FF) + 896 - wscale <= 2046;
   const double G = __hiloint2double((int)((unsigned)ghw + ((unsigned)(896 - wscale) << 20)), __double2loint(pp->g));
-  auto body = [&](auto fast_, auto gfold_, auto flush_) {
+  auto body = [&](auto fast_, auto gfold_, auto flush_, auto rag_) {
+    constexpr bool RAG = decltype(rag_)::value;   // the window holds a shorter last block
     constexpr bool FAST = decltype(fast_)::value;
     constexpr bool GFOLD = decltype(gfold_)::value;
     constexpr bool FLUSH = decltype(flush_)::value;
@@ -296,6 +321,13 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
         L[i] = ul;
       }
     }
+    if (RAG && ragt) {   // past the system's end u = 0, so that X = 0 reaches its last row
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        if (last0 && i >= nl) H[i].x = L[i].x = 0.f;
+        if (last1 && i >= nl) H[i].y = L[i].y = 0.f;
+      }
+    }
     {  // X_i = u_i + ib X_{i+1}, X_R = 0   (the particular solution is xp = g X)
       const float2 bh = f2(pp->ib_h), bl = f2(pp->ib_l);
       float2 xh = f2(0.f), xl = f2(0.f);
@@ -312,7 +344,22 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     // beta^L / g = K1 X_0 + K2 X_{n-1}, beta^R / g = K3 X_0 + K4 X_{n-1} (the block's beta record: the
     // 2x2 map M of eq. 16 applied to alpha / g = X_0 - ib v_0 X_0, omega / g = X_{n-1} - ib v_{n-1} X_0)
     const ff2 zero2{f2(0.f), f2(0.f)};
-    const ff2 X0 = ff2_make(H[0], L[0]), Xe = ff2_make(H[R - 1], L[R - 1]);
+    const ff2 X0 = ff2_make(H[0], L[0]);
+    float2 Xeh = H[R - 1], Xel = L[R - 1];
+    if (RAG && ragt) {
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        if (i == nl - 1) {
+          if (last0) {
+            Xeh.x = H[i].x;
+            Xel.x = L[i].x;
+          } else {
+            Xeh.y = H[i].y;
+            Xel.y = L[i].y;
+          }
+        }
+    }
+    const ff2 Xe = ff2_make(Xeh, Xel);
     // forward solve: the slot is idle until the output, so the 64 data registers wait there while
     // the tree runs.  Layout: the packed hi pair of row i (both blocks) at 8 i, the lo pair at
     // 8 R + 8 i, as the packed instructions take them; the output rows 2k, 2k+1 of block 2t go to
@@ -359,6 +406,8 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     const ff2 cR = ff2_pair(XR0, XR1);
     const float2 gh = f2(pp->g_h), glo = f2(pp->g_l);
     const double gd = pp->g;
+    const float4* sv4 = (RAG && ragt) ? rv4 : tv4;
+    const float4* sw4 = (RAG && ragt) ? rw4 : tw4;
 
     // the adjoint: x in the slots, its own power-of-two scale, the neighbours' boundary rows
     int xsc = 0;
@@ -466,7 +515,7 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
           xl = *reinterpret_cast<const float2*>(mine + 8 * R + 8 * i);
         }
         if (anyown) {
-          const float4 v = tv4[i], w = tw4[R - 1 - i];
+          const float4 v = sv4[i], w = sw4[R - 1 - i];
           ff_fma_acc2(cL.h, cL.l, make_float2(v.x, v.y), make_float2(v.z, v.w), xh, xl);
           ff_fma_acc2(cR.h, cR.l, make_float2(w.x, w.y), make_float2(w.z, w.w), xh, xl);
         }
@@ -527,7 +576,7 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
       }
     }
     __syncwarp();   // the warp's rows of x are in its slots
-    slots_store(smem, dst, hl * R, (hl + nown) * R, al_dst, lane, wid);
+    slots_store(smem, dst, hl * R, min(len, (hl + nown) * R), al_dst, lane, wid);
     if constexpr (ADJ) {
       // the CTA's three sums: the thread's own lanes, the warp, the CTA (fixed order), one join
       __syncthreads();   // the scan scratch takes the per-warp sums
@@ -576,14 +625,29 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
     else
       store_loop(std::false_type());
   };
-  if (fast && gfold)
-    body(std::true_type(), std::true_type(), std::false_type());
-  else if (flush && gfold)
-    body(std::true_type(), std::true_type(), std::true_type());
-  else if (fast)
-    body(std::true_type(), std::false_type(), std::false_type());
-  else
-    body(std::false_type(), std::false_type(), std::false_type());
+  const std::true_type yes;
+  const std::false_type no;
+  auto ragged = [&] {   // its own instantiations: the tests on rows would cost the others registers
+    if constexpr (RAGK) {
+      if (fast && gfold)
+        body(yes, yes, no, yes);
+      else if (flush && gfold)
+        body(yes, yes, yes, yes);
+      else
+        body(no, no, no, yes);
+    }
+  };
+  if (rag) {
+    ragged();
+  } else if (fast && gfold) {
+    body(yes, yes, no, no);
+  } else if (flush && gfold) {
+    body(yes, yes, yes, no);
+  } else if (fast) {
+    body(yes, no, no, no);
+  } else {
+    body(no, no, no, no);
+  }
 }
 
 }  // namespace dich
