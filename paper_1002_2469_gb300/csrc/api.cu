@@ -1496,6 +1496,22 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     const int sms = device_sms();
     if (w64 > 0 && w64 < 2 * (int64_t)sms) b->NT[FORM_F64] = 256;
   }
+  bool reg_rows = false;
+  if (o.n_req == 0 && !(o.flags & DICH_FLAG_SMEM_PATH)) {
+    int64_t longest = 0, nmix = 0, none = 0;   // MIXED windows, one-window systems among them
+    for (int64_t s = 0; s < nsys; ++s) {
+      if (h_N[s] < 8 * kRegRows || !std::isfinite(h_tm1[s]) || !std::isfinite(h_t0[s]) || !std::isfinite(h_tp1[s])) continue;
+      const Roots r = toeplitz_roots(h_tm1[s], h_t0[s], h_tp1[s]);
+      if (!r.ok || pick_form(o.prec, r) != FORM_MIXED) continue;
+      const int64_t w = ceil_div(h_N[s], (int64_t)window_blocks(default_threads(FORM_MIXED), FORM_MIXED) * kRegRows);
+      nmix += w;
+      none += (w == 1);
+      longest = std::max(longest, h_N[s]);
+    }
+    reg_rows = device_sms() > 0 && none >= 2 * (int64_t)device_sms() && 2 * none >= nmix;
+    // windows of half the width hold systems of up to 2048 rows
+    if (reg_rows && !o.NT && longest <= 128 * kRegRows) b->NT[FORM_MIXED] = 64;
+  }
   b->fwd.resize((size_t)nsys);
   b->adj.resize((size_t)nsys);
   b->form.assign((size_t)nsys, FORM_F64);
@@ -1527,7 +1543,14 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     }
     const int NTs = b->NT[b->form[s]];
     const int nmax = max_rows(NTs, b->form[s], o.n_req > 0 ? kSmemMax : kSmemBudget);
-    const int n = choose_n(h_N[s], window_blocks(NTs, b->form[s]), nmax, o.n_req, default_rows(b->form[s]));
+    int n = choose_n(h_N[s], window_blocks(NTs, b->form[s]), nmax, o.n_req, default_rows(b->form[s]));
+    // enough one-window MIXED systems to fill the chip and most of its windows: 16-row blocks for the register path, though they
+    // leave threads idle (shorter blocks, the choice for one system, go to the shared-memory path; from
+    // 12 rows on, in windows of full width, that is no slower): 2000 systems of 1822 rows 44.6 -> 26.0 us,
+    // 3000 of 700 41.2 -> 32.0, of 3000 rows 40.6 on either
+    if (reg_rows && b->form[s] == FORM_MIXED && n < (b->NT[FORM_MIXED] == 64 ? kRegRows : 12) &&
+        h_N[s] >= 8 * kRegRows && h_N[s] % kRegRows != 1)
+      n = kRegRows;
     Opts oh = o;
     oh.flags &= ~DICH_FLAG_FORCE_GENERAL;
     rc = build_system(h_tm1[s], h_t0[s], h_tp1[s], h_N[s], NTs, b->form[s], n, oh, true, b->fwd[s]);
@@ -1592,12 +1615,12 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
   if (b->ntf) b->ntf = fix_threads(b->NT[FORM_F64], b->n_smem[FORM_F64]);
   // MIXED windows take the register path wherever its shape allows (one-window systems too: 3946 Poisson
   // modes of 4096 rows 80.9 us, on the shared-memory path 93.0)
-  // -- in the kernel that also takes shorter last blocks where at least an eighth of the windows have one
+  // -- in the kernel that also takes shorter last blocks where at least half of the windows have one
   {
     int64_t rag = 0;
     for (int64_t s : order)
       if (b->form[s] == FORM_MIXED && b->fwd[s].rec.n == kRegRows && b->fwd[s].rec.nlast < kRegRows) ++rag;
-    b->reg_path = (o.flags & DICH_FLAG_SMEM_PATH) ? 0 : (8 * rag >= (int64_t)b->items[FORM_MIXED].size() && rag > 0) ? 2 : 1;
+    b->reg_path = (o.flags & DICH_FLAG_SMEM_PATH) ? 0 : (2 * rag >= (int64_t)b->items[FORM_MIXED].size() && rag > 0) ? 2 : 1;
   }
   // general-path systems: block offsets in the shared buffers, windows without halo, scan chunks
   for (int32_t s : b->general) {
