@@ -41,6 +41,8 @@ __device__ __forceinline__ Mat2 mat_norm(Mat2 m) {
   return Mat2{ldexp(m.a, 1 - e), ldexp(m.b, 1 - e), ldexp(m.c, 1 - e), ldexp(m.d, 1 - e)};
 }
 
+constexpr int kPreMaxes = 9;
+
 struct PreArgs {
   int64_t N, P;
   int n, nlast;
@@ -53,9 +55,10 @@ struct PreArgs {
   Mat2* fwd;            // per block: forward composite (rows s..e)
   Mat2* bwd;            // per block: backward composite (rows e..s)
   Mat2* chunk;          // 2 per chunk: forward, backward chunk products, then the incoming products
-  unsigned long long* maxes;   // [8]: bits of max |a_m| (m < P-1), max |c_m| (m > 0); a failure flag;
-                               // then for the precision choice: the largest forward and backward error
-                               // gains, max |rd_i|, ~bits of min |rd_i|, max |a_i|, |cp_i|, |v_i|, |w_i|
+  unsigned long long* maxes;   // [kPreMaxes]: bits of max |a_m| (m < P-1), max |c_m| (0 < m < P-1); a
+                               // failure flag; then for the precision choice: the largest forward and
+                               // backward error gains, max |rd_i|, ~bits of min |rd_i|, max |a_i|, |cp_i|,
+                               // |v_i|, |w_i|; the last block's |c_m|
 };
 
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(fabs(v)); }
@@ -259,7 +262,7 @@ __global__ void __launch_bounds__(kPreThreads) k_pre_records(const PreArgs A) {
                       isfinite(kL) && isfinite(kR);
   if (!finite) atomicOr(&A.maxes[2], 1ull);     // a zero pivot: the plan is refused as singular
   if (m < P - 1 && finite) atomicMax(&A.maxes[0], (unsigned long long)__double_as_longlong(fabs(pa)));
-  if (m > 0 && finite) atomicMax(&A.maxes[1], (unsigned long long)__double_as_longlong(fabs(pc)));
+  if (m > 0 && finite) atomicMax(&A.maxes[m < P - 1 ? 1 : 8], (unsigned long long)__double_as_longlong(fabs(pc)));
 }
 
 }  // namespace dich

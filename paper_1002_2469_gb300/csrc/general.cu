@@ -181,9 +181,15 @@ int gen_geometry(dich_gen_s* g, double b0) {
 }
 
 // windows: one window, halo windows (coupling beyond the halo below eps), or the general path,
-// from the largest |a| over blocks 0..P-2 and |c| over blocks 1..P-1 of the block maps
-void gen_decide(dich_gen_s* g, double amax, double cmax) {
-  g->gamma = std::max({1.0, amax, cmax});
+// from the largest |a| over blocks 0..P-2 and |c| over blocks 1..P-2 of the block maps.  The last
+// block's |c| (clast) stays out of the halos: a window that holds this block reaches the system's
+// end and has nothing beyond to truncate, and past any other window's end the coupling runs
+// through the window's own halo blocks, all of them full.  Its factor is that of a few rows in many
+// systems and would then set the halo for all: N = 8388613 ends in a block of 5 rows of 32, which
+// asked for 11 halo blocks to the right of 64-thread FP64 windows where the others need 3 (157 us
+// a solve; 134 without it).
+void gen_decide(dich_gen_s* g, double amax, double cmax, double clast) {
+  g->gamma = std::max({1.0, amax, cmax, clast});
   SysPlan& r = g->rec;
   const int64_t P = r.P;
   const int NT = g->NT;
@@ -259,7 +265,7 @@ int gen_host_tables(dich_gen_s* g, const double* a, const double* b, const doubl
   double* fv = g->rows.data() + GF_V * g->stride;
   double* fw = g->rows.data() + GF_W * g->stride;
   std::vector<double> lcp((size_t)n), lrd((size_t)n), z((size_t)n);
-  double amax = 0.0, cmax = 0.0;
+  double amax = 0.0, cmax = 0.0, clast = 0.0;
   for (int64_t m = 0; m < P; ++m) {
     const int64_t s = m * n;
     const int nb = (m == P - 1) ? r.nlast : n;
@@ -323,10 +329,11 @@ int gen_host_tables(dich_gen_s* g, const double* a, const double* b, const doubl
     rc[BC_M10] = -p10 / det;
     rc[BC_M11] = p00 / det;
     if (m < P - 1) amax = std::max(amax, std::fabs(pa));
-    if (m > 0) cmax = std::max(cmax, std::fabs(pc));
+    if (m > 0 && m < P - 1) cmax = std::max(cmax, std::fabs(pc));
+    if (m > 0 && m == P - 1) clast = std::fabs(pc);
   }
 
-  gen_decide(g, amax, cmax);
+  gen_decide(g, amax, cmax, clast);
   // precision form from the tables, then (MIXED) the tables as float-float pairs in place
   double fm = 1.0, bm = 1.0, rmax = 0.0, rmin = INFINITY, omax = 0.0;
   for (int64_t m = 0; m < P; ++m) {   // error gains of the two recurrences, block by block
@@ -422,22 +429,23 @@ int gen_device_tables(dich_gen_s* g, char* base, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(raw + N, g->hb.data(), nb, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(raw + 2 * N, g->hc.data(), nb, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(A.rows, 0, sizeof(double) * (size_t)(kGenFields * g->stride), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A.maxes, 0, 8 * sizeof(unsigned long long), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A.maxes, 0, kPreMaxes * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return cuda_fail(e);
   k_pre_blocks<<<(unsigned)nch, kPreThreads, 0, st>>>(A);
   k_pre_chunk<<<(unsigned)nch, kPreThreads, 0, st>>>(A);
   k_pre_top<<<1, 32, 0, st>>>(A, nch);
   k_pre_records<<<(unsigned)nch, kPreThreads, 0, st>>>(A);
   e = cudaGetLastError();
-  unsigned long long mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  unsigned long long mx[kPreMaxes] = {};
   if (e == cudaSuccess) e = cudaMemcpyAsync(mx, A.maxes, sizeof(mx), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e);
   if (mx[2]) return DICH_ERR_SINGULAR;
-  double amax, cmax;
+  double amax, cmax, clast;
   std::memcpy(&amax, &mx[0], sizeof(double));
   std::memcpy(&cmax, &mx[1], sizeof(double));
-  gen_decide(g, amax, cmax);
+  std::memcpy(&clast, &mx[8], sizeof(double));
+  gen_decide(g, amax, cmax, clast);
   double q[5];   // forward and backward error gains, max |rd|, min |rd|, max of the other factors
   mx[6] = ~mx[6];
   for (int j = 0; j < 5; ++j) std::memcpy(&q[j], &mx[3 + j], sizeof(double));

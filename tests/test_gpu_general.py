@@ -276,3 +276,29 @@ def test_residual_check_reports_what_it_sees(D):
     r, be = plan.residual(Fd, xd)
     rh, beh = host_residual(a, b, c, F, x)
     assert abs(be - beh) <= 1e-15 + 1e-3 * beh and plan.info["growth"] >= 1.0
+
+
+@pytest.mark.parametrize("prec", [0, 2])
+@pytest.mark.parametrize("prelim", [HOST, DEVICE])
+@pytest.mark.parametrize("nlast", [2, 3, 5, 31, 32])
+def test_general_short_last_block_leaves_the_halo_alone(D, nlast, prelim, prec):
+    """The last block (nlast rows of 32) does not widen the halos of the others, and what it holds
+    still reaches every window: its rows couple strongly (factors near 1) and carry right-hand sides
+    1e6 times the others'.  Several positions of the last window's start are met by the thread counts."""
+    N0 = 32 * 700
+    a, b, c = dominant(N0 + nlast, 21)
+    b = np.abs(b)
+    b[N0:] = np.abs(a[N0:]) + np.abs(c[N0:]) + 1e-3
+    F = np.random.default_rng(22).standard_normal(N0 + nlast)
+    F[N0:] *= 1e6
+    want = oracle.thomas_tridiag(a, b, c, F)
+    for threads in (64, 128):
+        kw = dict(flags=prelim, precision=prec, block_size=32, threads=threads)
+        _, full = gen_solve(D, a[:N0], b[:N0], c[:N0], F[:N0], **kw)
+        x, info = gen_solve(D, a, b, c, F, **kw)
+        assert (info["path"], info["halo_l"]) == (1, full["halo_l"])
+        # the shortened matrix ends in a full block of its own, which does not count either
+        assert abs(info["halo_r"] - full["halo_r"]) <= 1
+        # row by row: the exact solution decays from the last block's 1e6 into the others
+        assert np.max(np.abs(x - want)[:N0 - 640]) < TOL * np.max(np.abs(want[:N0 - 640]))
+        assert rel(x, want) < TOL, info
