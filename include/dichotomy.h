@@ -87,7 +87,8 @@ enum {
                                         check results with dichotomy_residual / dichotomy_gen_residual */
   /* MIXED-form window kernel of Toeplitz plans and batches (the results agree to rounding):
    * the register path keeps a thread's two 16-row blocks in registers; the shared-memory path sweeps
-   * the window's tile in shared memory.  Default: the register path wherever its shape allows. */
+   * the window's tile in shared memory.  Default: the register path wherever its shape allows, in
+   * batches if at least half of the windows have it. */
   DICH_FLAG_REG_PATH = 32,           /* the register path wherever its window shape allows */
   DICH_FLAG_SMEM_PATH = 64           /* the shared-memory path for every window */
 };

@@ -1484,33 +1484,63 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
   b->opts = o;
   for (int f = 0; f < 2; ++f) b->NT[f] = o.NT ? o.NT : default_threads(f);
   if (!o.NT && o.n_req == 0) {
-    // few FP64-form windows (a handful of ill-conditioned systems beside many MIXED ones, such as
-    // the lowest Poisson modes) are latency-bound: 256-thread windows of shorter blocks
+    // few FP64-form windows are latency-bound.  A batch of nothing else, all of its systems suited to
+    // the default windows (fixed point, or at most 16 rows a block), is fastest in these: 154 systems
+    // of 256 to 22682 rows 12.3 us a solve, in 256-thread windows 34.1; 32 of 4096 rows 8.5 and 14.1.
+    // A handful of ill-conditioned systems beside many MIXED ones (the lowest Poisson modes) takes
+    // 256-thread windows of shorter blocks: 300 modes of 2500 rows 17, else 47.
+    const int NTd = b->NT[FORM_F64];
+    const int sms = device_sms();
     int64_t w64 = 0;
+    bool mixed = false;
+    std::vector<int64_t> in64;
     for (int64_t s = 0; s < nsys; ++s) {
       if (h_N[s] < 2 || !std::isfinite(h_tm1[s]) || !std::isfinite(h_t0[s]) || !std::isfinite(h_tp1[s])) continue;
       const Roots r = toeplitz_roots(h_tm1[s], h_t0[s], h_tp1[s]);
-      if (r.ok && pick_form(o.prec, r) == FORM_F64)
-        w64 += ceil_div(h_N[s], (int64_t)default_threads(FORM_F64) * default_rows(FORM_F64));
+      if (!r.ok) continue;
+      if (pick_form(o.prec, r) != FORM_F64) {
+        mixed = true;
+        continue;
+      }
+      w64 += ceil_div(h_N[s], (int64_t)NTd * default_rows(FORM_F64));
+      if (w64 < 2 * (int64_t)sms) in64.push_back(s);
     }
-    const int sms = device_sms();
-    if (w64 > 0 && w64 < 2 * (int64_t)sms) b->NT[FORM_F64] = 256;
+    auto suits = [&](int64_t s) {
+      const int n = choose_n(h_N[s], NTd, max_rows(NTd, FORM_F64, kSmemBudget), 0, default_rows(FORM_F64));
+      SysBuild f, t;
+      Opts oh = o;
+      oh.flags &= ~DICH_FLAG_FORCE_GENERAL;
+      if (build_system(h_tm1[s], h_t0[s], h_tp1[s], h_N[s], NTd, FORM_F64, n, oh, true, f) != DICH_OK ||
+          build_system(h_tp1[s], h_t0[s], h_tm1[s], h_N[s], NTd, FORM_F64, n, oh, true, t) != DICH_OK)
+        return false;
+      if (f.path == PATH_GENERAL || t.path == PATH_GENERAL) return false;
+      if (std::max(f.rec.hl, t.rec.hl) + std::max(f.rec.hr, t.rec.hr) > NTd / 2) return false;
+      return n <= 16 || (f.rec.o_fix != 0 && t.rec.o_fix != 0);
+    };
+    if (w64 > 0 && w64 < 2 * (int64_t)sms && (mixed || !std::all_of(in64.begin(), in64.end(), suits)))
+      b->NT[FORM_F64] = 256;
   }
   bool reg_rows = false;
   if (o.n_req == 0 && !(o.flags & DICH_FLAG_SMEM_PATH)) {
-    int64_t longest = 0, nmix = 0, none = 0;   // MIXED windows, one-window systems among them
+    // one-window MIXED systems, enough to fill the chip, that fill windows of 2048 rows to three
+    // quarters: 16-row blocks for the register path though some threads idle.  Shorter blocks, one
+    // per thread, go to the shared-memory path; it is the slower one from here on (350 systems of
+    // 1822 rows 13.9 us and 10.5 on the register path, 2000 of 2048 30.4 and 23.1), and the faster
+    // one below, where the register path's 16 dependent rows are longer than a window needs (400 of
+    // 1000 8.5 and 11.1, 2000 of 500 20.8 and 24.2; 1500 rows: 600 systems 11.1 and 11.3)
+    int64_t nmix = 0, none = 0, rows = 0;   // MIXED windows, one-window systems among them
     for (int64_t s = 0; s < nsys; ++s) {
       if (h_N[s] < 8 * kRegRows || !std::isfinite(h_tm1[s]) || !std::isfinite(h_t0[s]) || !std::isfinite(h_tp1[s])) continue;
       const Roots r = toeplitz_roots(h_tm1[s], h_t0[s], h_tp1[s]);
       if (!r.ok || pick_form(o.prec, r) != FORM_MIXED) continue;
-      const int64_t w = ceil_div(h_N[s], (int64_t)window_blocks(default_threads(FORM_MIXED), FORM_MIXED) * kRegRows);
-      nmix += w;
-      none += (w == 1);
-      longest = std::max(longest, h_N[s]);
+      ++nmix;
+      if (h_N[s] <= 128 * kRegRows) {
+        ++none;
+        rows += h_N[s];
+      }
     }
-    reg_rows = device_sms() > 0 && none >= 2 * (int64_t)device_sms() && 2 * none >= nmix;
-    // windows of half the width hold systems of up to 2048 rows
-    if (reg_rows && !o.NT && longest <= 128 * kRegRows) b->NT[FORM_MIXED] = 64;
+    reg_rows = !o.NT && device_sms() > 0 && none >= 2 * (int64_t)device_sms() && none == nmix && rows >= none * 96 * kRegRows;
+    if (reg_rows) b->NT[FORM_MIXED] = 64;   // half the width: 2048 rows
   }
   b->fwd.resize((size_t)nsys);
   b->adj.resize((size_t)nsys);
@@ -1544,12 +1574,7 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     const int NTs = b->NT[b->form[s]];
     const int nmax = max_rows(NTs, b->form[s], o.n_req > 0 ? kSmemMax : kSmemBudget);
     int n = choose_n(h_N[s], window_blocks(NTs, b->form[s]), nmax, o.n_req, default_rows(b->form[s]));
-    // enough one-window MIXED systems to fill the chip and most of its windows: 16-row blocks for the register path, though they
-    // leave threads idle (shorter blocks, the choice for one system, go to the shared-memory path; from
-    // 12 rows on, in windows of full width, that is no slower): 2000 systems of 1822 rows 44.6 -> 26.0 us,
-    // 3000 of 700 41.2 -> 32.0, of 3000 rows 40.6 on either
-    if (reg_rows && b->form[s] == FORM_MIXED && n < (b->NT[FORM_MIXED] == 64 ? kRegRows : 12) &&
-        h_N[s] >= 8 * kRegRows && h_N[s] % kRegRows != 1)
+    if (reg_rows && b->form[s] == FORM_MIXED && n < kRegRows && h_N[s] >= 8 * kRegRows && h_N[s] % kRegRows != 1)
       n = kRegRows;
     Opts oh = o;
     oh.flags &= ~DICH_FLAG_FORCE_GENERAL;
@@ -1613,14 +1638,26 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     if (q.o_fix || b->adj[(size_t)s].rec.o_fix) b->ntf = 1;
   }
   if (b->ntf) b->ntf = fix_threads(b->NT[FORM_F64], b->n_smem[FORM_F64]);
-  // MIXED windows take the register path wherever its shape allows (one-window systems too: 3946 Poisson
-  // modes of 4096 rows 80.9 us, on the shared-memory path 93.0)
-  // -- in the kernel that also takes shorter last blocks where at least half of the windows have one
+  // MIXED windows take the register path where its shape allows (one-window systems too: 3946 Poisson
+  // modes of 4096 rows 80.9 us, on the shared-memory path 93.0), in the kernel that also takes
+  // shorter last blocks if such windows are no fewer than the others (600 systems of 5000 rows 30.7 us,
+  // else 37.4), in launches that keep the chip busy from half as many on (1500 systems of 2000 to
+  // 16384 rows 91.6 and 103.9; 310 of 256 to 16384 25.4 and 22.4).  With fewer than half of the
+  // windows of either kind the whole launch takes the shared-memory path, whose kernel alone is the
+  // faster one for the rest: 600 systems of 128 to 9000 rows 21.4 us, 23.9 in the register path's kernel
   {
-    int64_t rag = 0;
-    for (int64_t s : order)
-      if (b->form[s] == FORM_MIXED && b->fwd[s].rec.n == kRegRows && b->fwd[s].rec.nlast < kRegRows) ++rag;
-    b->reg_path = (o.flags & DICH_FLAG_SMEM_PATH) ? 0 : (2 * rag >= (int64_t)b->items[FORM_MIXED].size() && rag > 0) ? 2 : 1;
+    int64_t rag = 0, full = 0;
+    for (size_t i = 0; i < b->sys_ids[FORM_MIXED].size(); ++i) {
+      const SysPlan& q = b->fwd[(size_t)b->sys_ids[FORM_MIXED][i]].rec;
+      if (q.n != kRegRows) continue;
+      const int64_t last = q.nlast < kRegRows ? 1 : 0;
+      rag += last;
+      full += b->count[FORM_MIXED][i] - last;
+    }
+    const int64_t all = (int64_t)b->items[FORM_MIXED].size();
+    const bool ragged = rag >= full || (2 * rag >= full && all >= 12 * (int64_t)device_sms());
+    b->reg_path = ((o.flags & DICH_FLAG_SMEM_PATH) || 2 * (rag + full) < all) ? 0 : (ragged ? 2 : 1);
+    if (o.flags & DICH_FLAG_REG_PATH) b->reg_path = std::max(b->reg_path, 1);
   }
   // general-path systems: block offsets in the shared buffers, windows without halo, scan chunks
   for (int32_t s : b->general) {

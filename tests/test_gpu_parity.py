@@ -931,3 +931,28 @@ def test_cuda_graph_capture_of_a_batch(D):
         t = (tm1[s], t0[s], tp1[s])
         xq = oracle.thomas_q(t, F[sl])
         assert rel(x[sl].cpu().numpy(), xq) <= max(TOL, 20 * rel(oracle.thomas(t, F[sl]), xq)), s
+
+
+# (systems, shortest, longest, precision, weak): a few FP64 systems (in fixed-point windows of 4096 rows where
+# all of them suit it; one weakly dominant system keeps the wide windows), and 304 or more MIXED ones that
+# fill windows of 2048 rows to three quarters or just not
+@pytest.mark.parametrize("nsys,lo,hi,prec,weak", [(40, 2, 5000, 0, False), (40, 2, 5000, 0, True),
+                                                  (310, 1530, 1560, 1, False), (310, 1450, 2048, 1, False)])
+def test_batch_geometries(D, nsys, lo, hi, prec, weak):
+    rng = np.random.default_rng(nsys + lo)
+    N = rng.integers(lo, hi + 1, nsys)
+    N[:2] = lo, hi
+    off = W.offsets(N)
+    tm1, tp1 = rng.uniform(-1, -0.5, nsys), rng.uniform(-1, -0.5, nsys)
+    t0 = rng.uniform(2.05, 4, nsys)
+    if weak:
+        tm1[1], t0[1], tp1[1] = -1.0, 2.001, -1.0
+    F, w = rng.uniform(-1, 1, int(N.sum())), rng.uniform(-1, 1, int(N.sum()))
+    x, b = batch_solve(D, N, tm1, t0, tp1, F, precision=prec)
+    gF, _ = b.adjoint(torch.from_numpy(w).cuda(), torch.from_numpy(x).cuda())
+    ref = oracle.thomas_batched(tm1, t0, tp1, N, off, F)
+    lam = oracle.thomas_batched(tp1, t0, tm1, N, off, w)
+    gF = gF.cpu().numpy()
+    for o, n in zip(off, N):
+        assert rel(x[o:o + n], ref[o:o + n]) < TOL
+        assert rel(gF[o:o + n], lam[o:o + n]) < TOL
