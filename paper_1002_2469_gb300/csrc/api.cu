@@ -602,9 +602,10 @@ struct dich_plan_s {
   int64_t tiles = 0;
   SysBuild fwd, adj;
   // the default geometry of a plan that took a latency-bound one: many right-hand sides of a series
-  // fill the chip with it (wide.NT = 0: none)
+  // fill the chip with it (wide.NT = 0: none); from one right-hand side on, adjoints included, for weakly
+  // dominant systems of few windows
   struct {
-    SysBuild fwd;
+    SysBuild fwd, adj;
     int NT = 0, path = PATH_SINGLE, n_smem = 2, ntf = 0;
     int64_t tiles = 0, min_rhs = 0;    // taken from min_rhs right-hand sides on
   } wide;
@@ -662,11 +663,11 @@ static void plan_layout(dich_plan_s* p) {
   // workspace layout
   size_t o_ = 0;
   p->off_plans = o_;
-  o_ += align_up(3 * sizeof(SysPlan));
+  o_ += align_up(4 * sizeof(SysPlan));
   p->off_status = o_;
   o_ += kAlign;
   p->off_tabs = o_;
-  const size_t ntab = p->fwd.tab.size() + p->adj.tab.size() + p->corner.size() + p->wide.fwd.tab.size();
+  const size_t ntab = p->fwd.tab.size() + p->adj.tab.size() + p->corner.size() + p->wide.fwd.tab.size() + p->wide.adj.tab.size();
   o_ += align_up(sizeof(double) * ntab);
   const int64_t P = (p->N >= 2) ? p->fwd.rec.P : 0;
   if (p->path == PATH_GENERAL) {
@@ -678,17 +679,20 @@ static void plan_layout(dich_plan_s* p) {
     o_ += align_up(sizeof(double) * 6 * (size_t)ceil_div(P, kScanChunk));
   }
   p->off_part = o_;
-  o_ += align_up(sizeof(double) * 3 * (size_t)std::max<int64_t>(1, p->tiles));
+  o_ += align_up(sizeof(double) * 3 * (size_t)std::max<int64_t>({1, p->tiles, p->wide.tiles}));
   p->ws_bytes = o_;
   // staging copy: records, zero status, tables
   p->staging.assign(p->off_tabs + sizeof(double) * ntab, 0);
-  SysPlan recs[3] = {p->fwd.rec, p->adj.rec, p->wide.fwd.rec};
+  SysPlan recs[4] = {p->fwd.rec, p->adj.rec, p->wide.fwd.rec, p->wide.adj.rec};
   recs[0].tab = 0;
   recs[1].tab = (int64_t)p->fwd.tab.size();
   recs[2].tab = (int64_t)(p->fwd.tab.size() + p->adj.tab.size() + p->corner.size());
-  if (!p->wide.fwd.tab.empty())
-    std::memcpy(p->staging.data() + p->off_tabs + sizeof(double) * recs[2].tab, p->wide.fwd.tab.data(),
-                sizeof(double) * p->wide.fwd.tab.size());
+  recs[3].tab = recs[2].tab + (int64_t)p->wide.fwd.tab.size();
+  for (int i = 2; i < 4; ++i) {
+    const std::vector<double>& t = (i == 2) ? p->wide.fwd.tab : p->wide.adj.tab;
+    if (!t.empty())
+      std::memcpy(p->staging.data() + p->off_tabs + sizeof(double) * recs[i].tab, t.data(), sizeof(double) * t.size());
+  }
   std::memcpy(p->staging.data() + p->off_plans, recs, sizeof(recs));
   if (!p->fwd.tab.empty())
     std::memcpy(p->staging.data() + p->off_tabs, p->fwd.tab.data(), sizeof(double) * p->fwd.tab.size());
@@ -798,7 +802,10 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
     // fixed-point form one pass over overlapping windows is the faster way (tridiag{-1, 2.001, -1},
     // N = 2^24 + 1: 120 us against 348 us for the general path's two FP64 passes; solved in FP64, where
     // a window's values do not suit fixed point, such windows take about the general path's time).
-    // Only with a window for every SM: fewer of them leave SMs idle.
+    // A system with a window for every SM becomes a plan of such windows; a shorter one stays a plan of
+    // the general path (what its shards and its plan information are about) whose solves and adjoints
+    // of whole vectors take these windows too: N = 5894 to 752765 10 to 11 us, on the general path
+    // 78 to 82.
     if (o.NT == 0 && o.n_req == 0 && p->form == FORM_F64 && p->path == PATH_GENERAL &&
         !(o.flags & DICH_FLAG_FORCE_GENERAL)) {
       dich_plan_s q;
@@ -810,7 +817,17 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
       q.form = p->form;
       const int NT = 2 * p->NT;
       const int nc = choose_n(N, NT, max_rows(NT, p->form, kSmemBudget), 0, default_rows(p->form));
-      if (plan_geometry(&q, o, NT, nc) == DICH_OK && q.path == PATH_HALO && q.ntf && q.tiles >= device_sms()) {
+      const bool fits = plan_geometry(&q, o, NT, nc) == DICH_OK && q.path != PATH_GENERAL && q.ntf;
+      if (fits && (q.path != PATH_HALO || q.tiles < device_sms())) {
+        p->wide.NT = NT;
+        p->wide.fwd = std::move(q.fwd);
+        p->wide.adj = std::move(q.adj);
+        p->wide.path = q.path;
+        p->wide.n_smem = q.n_smem;
+        p->wide.ntf = q.ntf;
+        p->wide.tiles = q.tiles;
+        p->wide.min_rhs = 1;
+      } else if (fits) {
         p->NT = NT;
         p->fwd = std::move(q.fwd);
         p->adj = std::move(q.adj);
@@ -974,7 +991,9 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   // a series of enough right-hand sides to give every SM a window of the default geometry takes that
   // one (256 right-hand sides of 20011 rows, FP64 form: 36 us against 199.8 us with the plan's own
   // windows of 4-row blocks)
-  const bool wide = !adjoint && p->wide.NT != 0 && M >= p->wide.min_rhs;
+  // (a weakly dominant system of few windows always does, adjoints too)
+  const bool wide = p->wide.NT != 0 && M >= p->wide.min_rhs && (!adjoint || p->wide.min_rhs == 1);
+  const int path = wide ? p->wide.path : p->path;
   if (p->N == 1) {
     for (int64_t k = 0; k < M; ++k) {
       cudaError_t e = launch_trivial(d_plans, nullptr, 1, adjoint ? nullptr : F + k * ldf, x + k * ldx, xf,
@@ -994,12 +1013,12 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   a.part = adjoint ? (double*)(p->d_ws + p->off_part) : nullptr;
   a.check_finite = (p->opts.flags & DICH_FLAG_CHECK_FINITE) ? 1 : 0;
   a.n_smem = wide ? p->wide.n_smem : p->n_smem;
-  a.sys_offset = wide ? 2 : sys_offset;
+  a.sys_offset = (wide ? 2 : 0) + sys_offset;
   a.ldf = ldf;
   a.ldx = ldx;
   // the register path only for full solves of device memory, unless the plan asks
   // for the shared-memory path (the general path's passes always take that one)
-  a.reg_path = (device_mem && p->path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? 1 : 0;
+  a.reg_path = (device_mem && path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? 1 : 0;
   const int NT = wide ? p->wide.NT : p->NT, ntf = wide ? p->wide.ntf : p->ntf;
   const size_t smem = smem_bytes(NT, a.n_smem, p->form, ntf);
   // windows [win0, win0 + grid) of the single and halo paths (all of them unless a range is given)
@@ -1009,7 +1028,7 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
                                : launch_window_mixed(NT, grid, smem, st, w, gy);
   };
   cudaError_t e;
-  if (p->path != PATH_GENERAL) {
+  if (path != PATH_GENERAL) {
     // every right-hand side of a series in one launch (grid.y), at most 65535 per launch
     a.mode = MODE_FULL;
     a.win0 = win0;
@@ -1045,7 +1064,7 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
     if (e != cudaSuccess) return cuda_fail(e);
   }
   if (adjoint) {
-    e = launch_adj_finalize(a.part, nullptr, nullptr, nullptr, p->tiles, 1, gt, st);
+    e = launch_adj_finalize(a.part, nullptr, nullptr, nullptr, wide ? p->wide.tiles : p->tiles, 1, gt, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   if (p->quasi && adjoint) {
@@ -1061,7 +1080,7 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
     e = launch_end_gradients(xf, x, gt, p->N, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  if (p->quasi && !adjoint && !(p->path == PATH_GENERAL && M > 1)) {
+  if (p->quasi && !adjoint && !(path == PATH_GENERAL && M > 1)) {
     const double* ctab = d_tabs + p->fwd.tab.size() + p->adj.tab.size();
     CornerArgs c{p->N, p->Lg, p->Lh, ctab, ctab + p->Lg, p->psi, p->chi, p->W[0], p->W[1], p->W[2], p->W[3]};
     e = launch_corner(x, M, M > 1 ? ldx : 0, c, st);

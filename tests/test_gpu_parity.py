@@ -956,3 +956,34 @@ def test_batch_geometries(D, nsys, lo, hi, prec, weak):
     for o, n in zip(off, N):
         assert rel(x[o:o + n], ref[o:o + n]) < TOL
         assert rel(gF[o:o + n], lam[o:o + n]) < TOL
+
+
+@pytest.mark.parametrize("N", [4097, 5894, 8193, 16001, 300007])
+@pytest.mark.parametrize("t", [(-1.0, 2.001, -1.0), (0.9, 2.002, 1.1), (-1.0, 2.01, -0.98)])
+def test_weakly_dominant_systems_of_few_windows(D, t, N):
+    """Coupling longer than half a default window: the solve, the adjoint, a series, host vectors and corners,
+    which take fixed-point windows of twice the width where these hold it (one window of them, two,
+    or halo windows) and the general path where not."""
+    rng = np.random.default_rng(N)
+    F, w, G = rng.uniform(-1, 1, N), rng.uniform(-1, 1, N), rng.uniform(-1, 1, (3, N))
+    plan = D.Plan(*t, N, precision=0)
+    Fd = torch.from_numpy(F).cuda()
+    x = plan.solve(Fd)
+    xq = oracle.thomas_q(t, F)
+    assert rel(x.cpu().numpy(), xq) < TOL
+    gF, gt = plan.adjoint(torch.from_numpy(w).cuda(), x)
+    lam = oracle.thomas_q((t[2], t[1], t[0]), w)
+    assert rel(gF.cpu().numpy(), lam) < TOL
+    _, g = oracle.adjoint(t, w, xq)
+    assert np.max(np.abs(gt.cpu().numpy() - g)) < TOL * np.sum(np.abs(lam * xq))
+    xs = plan.solve_series(torch.from_numpy(G).cuda()).cpu().numpy()
+    for k in range(3):
+        assert rel(xs[k], oracle.thomas_q(t, G[k])) < TOL
+    assert rel(plan.solve_host(torch.from_numpy(F).pin_memory()).numpy(), xq) < TOL
+    quasi = D.Plan(*t, N, precision=0, psi=0.25, chi=-0.125)
+    y = quasi.solve(Fd).cpu().numpy()
+    a = np.full(N, t[0]); b = np.full(N, t[1]); c = np.full(N, t[2])
+    b[0] += 0.25
+    b[-1] -= 0.125
+    assert rel(y, oracle.thomas_tridiag(a, b, c, F)) < TOL
+    assert plan.status() == 0 and quasi.status() == 0
