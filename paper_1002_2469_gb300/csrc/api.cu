@@ -994,6 +994,7 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   // (a weakly dominant system of few windows always does, adjoints too)
   const bool wide = p->wide.NT != 0 && M >= p->wide.min_rhs && (!adjoint || p->wide.min_rhs == 1);
   const int path = wide ? p->wide.path : p->path;
+  const SysPlan& rec = wide ? p->wide.fwd.rec : p->fwd.rec;
   if (p->N == 1) {
     for (int64_t k = 0; k < M; ++k) {
       cudaError_t e = launch_trivial(d_plans, nullptr, 1, adjoint ? nullptr : F + k * ldf, x + k * ldx, xf,
@@ -1017,8 +1018,12 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   a.ldf = ldf;
   a.ldx = ldx;
   // the register path only for full solves of device memory, unless the plan asks
-  // for the shared-memory path (the general path's passes always take that one)
-  a.reg_path = (device_mem && path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? 1 : 0;
+  // for the shared-memory path (the general path's passes always take that one); up to some 14000
+  // windows (5.6e7 rows) in the kernel that also takes a shorter last block if there is one: the
+  // shared-memory path's window, the last to start, would end long after the others (N = 752765
+  // 14.4 us, here 9.6; 5000005 30.5 and 24.7; 64000005 230 on either; 200000005 675 and 690)
+  const int ragged = (rec.nlast < rec.n && (wide ? p->wide.tiles : p->tiles) <= 14000) ? 2 : 1;
+  a.reg_path = (device_mem && path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? ragged : 0;
   const int NT = wide ? p->wide.NT : p->NT, ntf = wide ? p->wide.ntf : p->ntf;
   const size_t smem = smem_bytes(NT, a.n_smem, p->form, ntf);
   // windows [win0, win0 + grid) of the single and halo paths (all of them unless a range is given)
