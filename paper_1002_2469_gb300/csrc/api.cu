@@ -1018,11 +1018,12 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   a.ldf = ldf;
   a.ldx = ldx;
   // the register path only for full solves of device memory, unless the plan asks
-  // for the shared-memory path (the general path's passes always take that one); up to some 14000
-  // windows (5.6e7 rows) in the kernel that also takes a shorter last block if there is one: the
-  // shared-memory path's window, the last to start, would end long after the others (N = 752765
-  // 14.4 us, here 9.6; 5000005 30.5 and 24.7; 64000005 230 on either; 200000005 675 and 690)
-  const int ragged = (rec.nlast < rec.n && (wide ? p->wide.tiles : p->tiles) <= 14000) ? 2 : 1;
+  // for the shared-memory path (the general path's passes always take that one).  A shorter last block
+  // puts the last window on that path, which takes longer than the others: launches whose windows
+  // all run at once take the kernel that has such blocks on the register path too (N = 752765 10.1 us,
+  // without it 14.9); with more windows it hides behind the others, as the first to start, and the
+  // plain kernel is the faster one (N = 4000005 20.6 us and 21.4, 32000005 117.0 and 122.7)
+  const int ragged = (rec.nlast < rec.n && (wide ? p->wide.tiles : p->tiles) <= kRagWindows) ? 2 : 1;
   a.reg_path = (device_mem && path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? ragged : 0;
   const int NT = wide ? p->wide.NT : p->NT, ntf = wide ? p->wide.ntf : p->ntf;
   const size_t smem = smem_bytes(NT, a.n_smem, p->form, ntf);

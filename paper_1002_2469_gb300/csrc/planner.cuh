@@ -13,6 +13,7 @@ namespace dich {
 namespace plan {
 
 constexpr size_t kAlign = 256;
+constexpr int64_t kRagWindows = 768;   // MIXED windows that run at once (five CTAs on each SM)
 // shared-memory budget per CTA for library-chosen block sizes (several CTAs share an SM so
 // the load, sweeps, tree and store of different windows overlap)
 constexpr size_t kSmemBudget = 110 * 1024;

@@ -33,7 +33,7 @@ namespace dich {
 struct WinArgs {
   const SysPlan* plans;   // plan records (device)
   const double* tabs;     // table buffer (device)
-  const Item* items;      // batched: one item per CTA; nullptr: single system, window = blockIdx
+  const Item* items;      // batched: one item per CTA; nullptr: single system, one window per CTA
   const double* F;        // right-hand sides
   double* x;              // solutions
   unsigned* status;       // device status word
@@ -46,7 +46,7 @@ struct WinArgs {
   int32_t n_smem;         // shared-memory rows (>= largest block size in the launch)
   int32_t sys_offset;     // added to the item's system index (adjoint twin records)
   int64_t ldf, ldx;       // series: right-hand side blockIdx.y starts at F + y ldf, its solution at x + y ldx
-  int64_t win0;           // single system: window of CTA blockIdx.x is win0 + blockIdx.x
+  int64_t win0;           // single system: the launch's windows are win0 + [0, gridDim.x)
   int32_t reg_path;       // F and x are device memory: windows of the register path's shape may take it
                           // (2: also those with a shorter last block)
 };

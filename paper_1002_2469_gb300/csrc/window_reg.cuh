@@ -154,6 +154,12 @@ __device__ __forceinline__ void tree_mid(const float2* tf, int rm, int pw, const
   if (b1 + 1 < nwin) XR1 = xs_next;
 }
 
+// a CTA's place among the gradient partials: its window's index (single systems run the last window
+// first), or its item's
+__device__ __forceinline__ unsigned part_of(const WinArgs& A) {
+  return A.items ? blockIdx.x : gridDim.x - 1 - blockIdx.x;
+}
+
 // ADJ: the adjoint (a5) -- A.F is w, the plan the transposed one, A.x receives lambda, and the
 // gradient sums -(sum lambda_r x_{r-1}, sum lambda_r x_r, sum lambda_r x_{r+1}) over the window's own
 // rows go to A.part (three per CTA).  The forward solution x (A.xf) comes into the pair slots by a
@@ -598,7 +604,7 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
           ffv sum = ff_zero();
           for (int w = 0; w < NW; ++w) sum = ff_add(sum, swv[tid * NW + w]);
           // lambda = g X 2^-wscale, x = x' 2^-xscale
-          A.part[3 * (size_t)blockIdx.x + tid] = join_dadd(sum.h, sum.l, xsc) * pow2i(-wscale) * gd;
+          A.part[3 * (size_t)part_of(A) + tid] = join_dadd(sum.h, sum.l, xsc) * pow2i(-wscale) * gd;
         }
       } else {
         double a3[3] = {(own0 ? dm0 : 0.0) + (own1 ? dm1 : 0.0), (own0 ? d00 : 0.0) + (own1 ? d01 : 0.0),
@@ -615,7 +621,7 @@ __device__ __forceinline__ void window_reg(const WinArgs& A, const SysPlan* pp, 
         if (tid < 3) {
           double sum = 0.0;
           for (int w = 0; w < NW; ++w) sum += sred[tid * NW + w];
-          A.part[3 * (size_t)blockIdx.x + tid] = sum;
+          A.part[3 * (size_t)part_of(A) + tid] = sum;
         }
       }
     }
