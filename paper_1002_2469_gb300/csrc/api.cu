@@ -1508,6 +1508,7 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
   b->nsys = nsys;
   b->opts = o;
   for (int f = 0; f < 2; ++f) b->NT[f] = o.NT ? o.NT : default_threads(f);
+  std::vector<std::pair<SysBuild, SysBuild>> built;
   if (!o.NT && o.n_req == 0) {
     // few FP64-form windows are latency-bound.  A batch of nothing else, all of its systems suited to
     // the default windows (fixed point, or at most 16 rows a block), is fastest in these: 154 systems
@@ -1530,20 +1531,23 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
       w64 += ceil_div(h_N[s], (int64_t)NTd * default_rows(FORM_F64));
       if (w64 < 2 * (int64_t)sms) in64.push_back(s);
     }
-    auto suits = [&](int64_t s) {
-      const int n = choose_n(h_N[s], NTd, max_rows(NTd, FORM_F64, kSmemBudget), 0, default_rows(FORM_F64));
-      SysBuild f, t;
-      Opts oh = o;
-      oh.flags &= ~DICH_FLAG_FORCE_GENERAL;
-      if (build_system(h_tm1[s], h_t0[s], h_tp1[s], h_N[s], NTd, FORM_F64, n, oh, true, f) != DICH_OK ||
-          build_system(h_tp1[s], h_t0[s], h_tm1[s], h_N[s], NTd, FORM_F64, n, oh, true, t) != DICH_OK)
-        return false;
-      if (f.path == PATH_GENERAL || t.path == PATH_GENERAL) return false;
-      if (std::max(f.rec.hl, t.rec.hl) + std::max(f.rec.hr, t.rec.hr) > NTd / 2) return false;
-      return n <= 16 || (f.rec.o_fix != 0 && t.rec.o_fix != 0);
-    };
-    if (w64 > 0 && w64 < 2 * (int64_t)sms && (mixed || !std::all_of(in64.begin(), in64.end(), suits)))
-      b->NT[FORM_F64] = 256;
+    if (w64 > 0 && w64 < 2 * (int64_t)sms && !mixed) {
+      built.resize((size_t)nsys);   // the default windows' plans, kept if every system suits them
+      auto suits = [&](int64_t s) {
+        const int n = choose_n(h_N[s], NTd, max_rows(NTd, FORM_F64, kSmemBudget), 0, default_rows(FORM_F64));
+        SysBuild &f = built[(size_t)s].first, &t = built[(size_t)s].second;
+        Opts oh = o;
+        oh.flags &= ~DICH_FLAG_FORCE_GENERAL;
+        if (build_system(h_tm1[s], h_t0[s], h_tp1[s], h_N[s], NTd, FORM_F64, n, oh, true, f) != DICH_OK ||
+            build_system(h_tp1[s], h_t0[s], h_tm1[s], h_N[s], NTd, FORM_F64, n, oh, true, t) != DICH_OK)
+          return false;
+        if (f.path == PATH_GENERAL || t.path == PATH_GENERAL) return false;
+        if (std::max(f.rec.hl, t.rec.hl) + std::max(f.rec.hr, t.rec.hr) > NTd / 2) return false;
+        return n <= 16 || (f.rec.o_fix != 0 && t.rec.o_fix != 0);
+      };
+      if (!std::all_of(in64.begin(), in64.end(), suits)) built.clear();
+    }
+    if (w64 > 0 && w64 < 2 * (int64_t)sms && built.empty()) b->NT[FORM_F64] = 256;
   }
   bool reg_rows = false;
   if (o.n_req == 0 && !(o.flags & DICH_FLAG_SMEM_PATH)) {
@@ -1603,8 +1607,13 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
       n = kRegRows;
     Opts oh = o;
     oh.flags &= ~DICH_FLAG_FORCE_GENERAL;
-    rc = build_system(h_tm1[s], h_t0[s], h_tp1[s], h_N[s], NTs, b->form[s], n, oh, true, b->fwd[s]);
-    if (!rc) rc = build_system(h_tp1[s], h_t0[s], h_tm1[s], h_N[s], NTs, b->form[s], n, oh, true, b->adj[s]);
+    if (!built.empty() && built[(size_t)s].first.rec.N == h_N[s]) {
+      b->fwd[s] = std::move(built[(size_t)s].first);
+      b->adj[s] = std::move(built[(size_t)s].second);
+    } else {
+      rc = build_system(h_tm1[s], h_t0[s], h_tp1[s], h_N[s], NTs, b->form[s], n, oh, true, b->fwd[s]);
+      if (!rc) rc = build_system(h_tp1[s], h_t0[s], h_tm1[s], h_N[s], NTs, b->form[s], n, oh, true, b->adj[s]);
+    }
     if (rc) {
       delete b;
       return rc;
