@@ -147,9 +147,17 @@ namespace {
 // prefers 32-row blocks in 64-thread windows; the float-float kernel, bound by the latency of its
 // coefficient loads, prefers 16-row blocks in 128-thread windows (more warps per SM).  AUTO plans
 // take the float-float geometry, as they usually run in that form.
+// Short FP64 systems leave the chip short of windows: up to kGenShortRows rows they take the
+// float-float geometry, windows of as many rows in twice the warps (N = 100003 16.5 us a solve, so
+// 10.5; 400000 15.6 and 14.2; from 8e5 rows on 19.6 and 22.1).
 constexpr int kGenDefaultRows = 32;
+constexpr int64_t kGenShortRows = 1 << 19;
 constexpr int kGenDefaultRowsFF = 16;
 constexpr int64_t kGenDevicePrelimMin = 1 << 15;   // default: device preliminary from this many rows
+
+bool gen_short(int64_t N, const Opts& o) {
+  return o.prec == DICH_PREC_F64 && o.NT == 0 && o.n_req == 0 && N <= kGenShortRows;
+}
 
 // block geometry (block size n, P blocks, the last one nlast rows); returns a status code
 int gen_geometry(dich_gen_s* g, double b0) {
@@ -163,7 +171,8 @@ int gen_geometry(dich_gen_s* g, double b0) {
   const size_t budget = g->opts.n_req > 0 ? kSmemMax : kSmemBudget;
   int nmax = 2;
   while (window_gen_smem_bytes(NT, nmax + 1) <= budget) ++nmax;
-  const int n = choose_n(N, NT, nmax, g->opts.n_req, g->opts.prec == DICH_PREC_F64 ? kGenDefaultRows : kGenDefaultRowsFF);
+  const int n = choose_n(N, NT, nmax, g->opts.n_req,
+                         g->opts.prec == DICH_PREC_F64 && !gen_short(g->N, g->opts) ? kGenDefaultRows : kGenDefaultRowsFF);
   const int64_t P = ceil_div(N, n);
   r.n = n;
   r.P = P;
@@ -204,7 +213,8 @@ void gen_decide(dich_gen_s* g, double amax, double cmax, double clast) {
   if (P <= NT) {
     g->path = PATH_SINGLE;
     r.own = (int32_t)P;
-  } else if (!(g->opts.flags & DICH_FLAG_FORCE_GENERAL) && hl + hr <= NT / 2) {
+  } else if (!(g->opts.flags & DICH_FLAG_FORCE_GENERAL) && hl + hr <= (gen_short(g->N, g->opts) ? 5 * NT / 8 : NT / 2)) {
+    // (5/8: halos of 16-row blocks can be a few more than twice those of 32 rows)
     g->path = PATH_HALO;
     r.hl = (int32_t)hl;
     r.hr = (int32_t)hr;
@@ -542,7 +552,7 @@ int dichotomy_gen_plan(int64_t N, const double* h_a, const double* h_b, const do
   if (!g) return DICH_ERR_ARG;
   g->N = N;
   g->opts = o;
-  g->NT = o.NT ? o.NT : (o.prec == DICH_PREC_F64 ? 64 : 128);
+  g->NT = o.NT ? o.NT : (o.prec == DICH_PREC_F64 && !gen_short(N, o) ? 64 : 128);
   g->norm_inf = norm_inf;
   if (N >= 1) {
     rc = gen_geometry(g, h_b[0]);

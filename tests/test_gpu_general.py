@@ -302,3 +302,17 @@ def test_general_short_last_block_leaves_the_halo_alone(D, nlast, prelim, prec):
         # row by row: the exact solution decays from the last block's 1e6 into the others
         assert np.max(np.abs(x - want)[:N0 - 640]) < TOL * np.max(np.abs(want[:N0 - 640]))
         assert rel(x, want) < TOL, info
+
+
+@pytest.mark.parametrize("N", [2047, 2049, 4096, 65537, (1 << 19) - 1, 1 << 19, (1 << 19) + 1])
+@pytest.mark.parametrize("margin", [(0.05, 2.0), (0.008, 0.012)])
+def test_general_fp64_default_geometry(D, N, margin):
+    """FP64 plans on both sides of the length where the default geometry changes, with halos of a
+    few blocks and of more than half a window."""
+    rng = np.random.default_rng(N)
+    a, c = -rng.uniform(0.9, 1.0, N), -rng.uniform(0.9, 1.0, N)
+    b = np.abs(a) + np.abs(c) + rng.uniform(*margin, N)
+    F = rng.standard_normal(N)
+    x, info = gen_solve(D, a, b, c, F, precision=0)
+    assert info["n"] == (32 if N > 1 << 19 else 16) or N == 2047 or N % 16 == 1
+    assert rel(x, oracle.thomas_tridiag(a, b, c, F)) < TOL
