@@ -260,8 +260,11 @@ static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
 // 50-row blocks ran at half speed).  A last block of a single row is not allowed (Sec. 2.1
 // asks for sub-vectors of >= 2 rows), so n moves to the nearest size with N mod n != 1:
 // upwards when the system fits in one window (every larger n still does), else downwards first.
-int choose_n(int64_t N, int NT, int nmax, int n_req, int n_def) {
-  auto ok = [&](int64_t c) { return c >= 2 && (c >= N || N % c != 1); };
+// one_row: the MIXED form's default blocks of 16 rows may leave a last block of a single row.  (Its
+// formulas hold for one row -- alpha = omega, M maps both to alpha / (1 - kL v_0) -- and 15- or 17-row
+// blocks would take every window off the register path: N = 3000001 27.9 us, here 17.4.)
+int choose_n(int64_t N, int NT, int nmax, int n_req, int n_def, bool one_row) {
+  auto ok = [&](int64_t c) { return c >= 2 && (c >= N || N % c != 1 || (one_row && c == kRegRows)); };
   const bool one_window = (n_req <= 0) && (N <= (int64_t)NT * std::min(nmax, n_def));
   int n;
   if (n_req > 0)
@@ -293,7 +296,7 @@ int build_system(double tm1, double t0, double tp1, int64_t N, int NT, int form,
   p.n = n;
   p.P = ceil_div(N, n);
   p.nlast = (int)(N - (p.P - 1) * (int64_t)n);
-  if (p.nlast < 2) return DICH_ERR_ARG;  // guarded by choose_n
+  if (p.nlast < 2 && form != FORM_MIXED) return DICH_ERR_ARG;  // guarded by choose_n
   p.form = form;
   p.tm1 = tm1;
   p.t0 = t0;
@@ -786,7 +789,7 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
   if (N >= 2) {
     const int n0 = choose_n(N, window_blocks(p->NT, p->form),
                             max_rows(p->NT, p->form, o.n_req > 0 ? kSmemMax : kSmemBudget), o.n_req,
-                            default_rows(p->form));
+                            default_rows(p->form), p->form == FORM_MIXED && o.n_req == 0);
     rc = plan_geometry(p, o, p->NT, n0);
     if (rc) {
       delete p;
@@ -856,7 +859,7 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
         q.tp1 = t_1;
         q.opts = o;
         q.form = p->form;
-        const int nc = choose_n(N, window_blocks(NT, p->form), max_rows(NT, p->form, kSmemBudget), n, n);
+        const int nc = choose_n(N, window_blocks(NT, p->form), max_rows(NT, p->form, kSmemBudget), n, n, p->form == FORM_MIXED);
         if (plan_geometry(&q, o, NT, nc) != DICH_OK || q.path != PATH_HALO) break;
         if (p->wide.NT == 0) {
           p->wide.NT = p->NT;
@@ -1602,8 +1605,8 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     }
     const int NTs = b->NT[b->form[s]];
     const int nmax = max_rows(NTs, b->form[s], o.n_req > 0 ? kSmemMax : kSmemBudget);
-    int n = choose_n(h_N[s], window_blocks(NTs, b->form[s]), nmax, o.n_req, default_rows(b->form[s]));
-    if (reg_rows && b->form[s] == FORM_MIXED && n < kRegRows && h_N[s] >= 8 * kRegRows && h_N[s] % kRegRows != 1)
+    int n = choose_n(h_N[s], window_blocks(NTs, b->form[s]), nmax, o.n_req, default_rows(b->form[s]), b->form[s] == FORM_MIXED && o.n_req == 0);
+    if (reg_rows && b->form[s] == FORM_MIXED && n < kRegRows && h_N[s] >= 8 * kRegRows)
       n = kRegRows;
     Opts oh = o;
     oh.flags &= ~DICH_FLAG_FORCE_GENERAL;

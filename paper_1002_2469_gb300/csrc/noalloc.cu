@@ -101,7 +101,7 @@ extern "C" int dichotomy_solve_noalloc(double t_m1, double t_0, double t_1, int6
   int n = 2;
   if (N >= 2) {
     const int nmax = max_rows(NT, form, kSmemBudget);
-    n = choose_n(N, window_blocks(NT, form), nmax, 0, default_rows(form));
+    n = choose_n(N, window_blocks(NT, form), nmax, 0, default_rows(form), form == FORM_MIXED);
     rc = build_system(t_m1, t_0, t_1, N, NT, form, n, o, true, sb);
     if (rc) return rc;                                  // DICH_ERR_WORKSPACE: tables exceed the array
   } else {

@@ -57,7 +57,7 @@ int validate_t(double tm1, double t0, double tp1, int flags = 0);
 int read_opts(const dich_opts* o, Opts& out);
 int pick_form(int prec, const Roots& r);
 int64_t ceil_div(int64_t a, int64_t b);
-int choose_n(int64_t N, int NT, int nmax, int n_req, int n_def);
+int choose_n(int64_t N, int NT, int nmax, int n_req, int n_def, bool one_row = false);
 int build_system(double tm1, double t0, double tp1, int64_t N, int NT, int form, int n, const Opts& o,
                  bool allow_general, SysBuild& sb);
 bool is_device_ptr(const void* p);

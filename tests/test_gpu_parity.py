@@ -987,3 +987,28 @@ def test_weakly_dominant_systems_of_few_windows(D, t, N):
     b[-1] -= 0.125
     assert rel(y, oracle.thomas_tridiag(a, b, c, F)) < TOL
     assert plan.status() == 0 and quasi.status() == 0
+
+
+@pytest.mark.parametrize("N", [3841, 3857, 4097, 4113, 600001, 3300001])
+@pytest.mark.parametrize("flags", [0, 1, 64])
+def test_mixed_last_block_of_one_row(D, N, flags):
+    """Lengths 16 k + 1 in the MIXED form: 16-row blocks with one row left over, alone in its block
+    (first or second of a thread's pair), on the register, shared-memory and general paths."""
+    t = (-1.2, 2.5, -0.8)
+    rng = np.random.default_rng(N)
+    F, w = rng.uniform(-1, 1, N), rng.uniform(-1, 1, N)
+    plan = D.Plan(*t, N, precision=1, flags=flags)
+    x = plan.solve(torch.from_numpy(F).cuda())
+    gF, gt = plan.adjoint(torch.from_numpy(w).cuda(), x)
+    x, ref = x.cpu().numpy(), oracle.thomas(t, F)
+    assert rel(x, ref) < TOL and abs(x[-1] - ref[-1]) < TOL, plan.info
+    lam, g = oracle.adjoint(t, w, ref)
+    assert rel(gF.cpu().numpy(), lam) < TOL
+    assert np.max(np.abs(gt.cpu().numpy() - g)) < TOL * np.sum(np.abs(lam * ref))
+    Ns = np.array([N, 4097, 3873, 20001])
+    Fb = rng.uniform(-1, 1, int(Ns.sum()))
+    tm1, t0, tp1 = np.full(4, t[0]), np.full(4, t[1]), np.full(4, t[2])
+    y, _ = batch_solve(D, Ns, tm1, t0, tp1, Fb, precision=1, flags=flags & 64)
+    ref = oracle.thomas_batched(tm1, t0, tp1, Ns, W.offsets(Ns), Fb)
+    assert np.max(np.abs(y - ref)) < TOL * np.max(np.abs(ref))
+    assert plan.status() == 0
