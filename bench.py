@@ -376,7 +376,7 @@ def run_gpu(args):
         "fp64_plain": {"value": round(world * N / (f64_ms * 1e-3) / 1e9, 3), "unit": "Gunknowns/s",
                        "ms_per_step": round(f64_ms, 5), "rel_err_vs_oracle": f64["rel_err"],
                        "backward_err": f64["backward_err"],
-                       "bound": "alu (FP64 pipe)", "block_size": f64["info"]["n"],
+                       "bound": "integer multiply and FP64 pipes (64-bit fixed point)", "block_size": f64["info"]["n"],
                        "threads_per_window": f64["info"]["threads"], "device_status": f64["status"]},
         "roofline": {"bound": _bound(kernel_key, "unprofiled"), "achieved": round(achieved, 1), "peak": peak,
                      "unit": "GB/s",
@@ -610,8 +610,8 @@ def other_configs(D, W, oracle, stream, world, steps=10, only=None, cpu_leg=True
         if c4_systems:   # the first systems only (a smaller case of the same series, for profiling)
             N, off_tight, tm1, t0, tp1 = N[:c4_systems], off_tight[:c4_systems], tm1[:c4_systems], \
                 t0[:c4_systems], tp1[:c4_systems]
-        # layout: every system at a 16-byte aligned offset (even row), where the register path's bulk
-        # copies can start; the tightly packed layout (odd offsets after odd sizes) is timed beside it
+        # layout: every system at a 16-byte aligned offset (even row), where the register path copies
+        # 16 bytes at a time; the tightly packed layout (odd offsets: 8-byte copies) is timed beside it
         off = W.offsets(N + (N & 1))
         Fd = W.device_uniform(int(off[-1] + N[-1]), W.SEED_RHS, "cuda")
         xd = torch.empty_like(Fd)
@@ -632,7 +632,7 @@ def other_configs(D, W, oracle, stream, world, steps=10, only=None, cpu_leg=True
                 mst = _time_batch(lambda: bt.solve(Fd, out=xd), max(3, steps // 2), world, stream)
                 c4["auto_tight_layout"] = {"ms": round(mst, 3), "Gunknowns_s": round(N.sum() / mst / 1e6, 2),
                                            "odd_offsets": int((off_tight & 1).sum()),
-                                           "note": "systems at odd offsets take the shared-memory path"}
+                                           "note": "systems at odd offsets: 8-byte copies"}
                 del bt
         if cpu_leg:
             nh = int(np.searchsorted(np.cumsum(N), 1 << 28) + 1)      # the first ~2 GB of systems
@@ -689,7 +689,7 @@ def other_configs(D, W, oracle, stream, world, steps=10, only=None, cpu_leg=True
         u = solver.solve(fd).cpu().numpy()
         out["f3_poisson2d_4095"] = {"unknowns": M * M, "ms_total": round(ms_total, 4), "ms_dichotomy": round(ms_solve, 4),
                                     "Gunknowns_s": round(M * M / ms_total / 1e6, 2),
-                                    "form": "AUTO per mode", "transform": "DST-I via torch.fft (cuFFT)",
+                                    "form": "AUTO per mode", "transform": "DST-I, FFT in 64-bit fixed point",
                                     "rel_err_vs_manufactured": float(np.max(np.abs(u - us)) / np.max(np.abs(us)))}
         del fd, rhs, v, solver
         torch.cuda.empty_cache()

@@ -257,8 +257,8 @@ static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
 // blocks (n = ceil(N / window blocks) <= n_def), else n_def rows per block.  Longer blocks
 // would fit one window up to nmax rows, but they serialise the sweeps and enlarge the shared
 // memory of every CTA of a batched launch (measured: a batch with some one-window systems of
-// 50-row blocks ran at half speed).  A last block of a single row is not allowed (Sec. 2.1
-// asks for sub-vectors of >= 2 rows), so n moves to the nearest size with N mod n != 1:
+// 50-row blocks ran at half speed).  A last block of a single row is avoided (Sec. 2.1
+// asks for sub-vectors of >= 2 rows; but see one_row), so n moves to the nearest size with N mod n != 1:
 // upwards when the system fits in one window (every larger n still does), else downwards first.
 // one_row: the MIXED form's default blocks of 16 rows may leave a last block of a single row.  (Its
 // formulas hold for one row -- alpha = omega, M maps both to alpha / (1 - kL v_0) -- and 15- or 17-row

@@ -306,13 +306,15 @@ __host__ __device__ inline size_t window2_smem_bytes(int NT, int n_smem) {
 
 // Instantiations: KIND_REG -- the forward solve with the register path for windows it serves (up to
 // 80 registers: six CTAs of 128 threads per SM); KIND_SMEM -- the forward solve on the shared-memory
-// path only (80 registers: six CTAs per SM, for launches of many short, latency-bound windows);
+// path only (80 registers: six CTAs per SM; launches that ask for it, mapped host memory, the general
+// path's passes, batches with fewer than half of their windows on the register path);
 // KIND_ADJ -- the adjoint (shared-memory path, gradient sums in the store loop, six CTAs per SM).
 // KIND_REGADJ -- the adjoint with the register path for the windows it serves (up to 128 registers:
 // four CTAs per SM; its slots hold x during the tree).
-// KIND_REGRAG -- KIND_REG with the register path also for windows whose last block is shorter, for launches
-// where many windows are of that kind (4000 systems of 4095 rows: 96 us against 147); where few are, the
-// larger kernel costs more than they gain (2^26 rows 231 -> 240 us, 1500 uneven systems 830 -> 864).
+// KIND_REGRAG -- KIND_REG with the register path also for windows whose last block is shorter, for batches
+// where many windows are of that kind (4000 systems of 4095 rows: 96 us against 147) and single systems
+// whose windows all run at once; elsewhere the larger kernel costs more than they gain (N = 32000005
+// 117.0 -> 122.7 us, 1500 uneven systems 830 -> 864).
 enum WinKind : int { KIND_REG = 0, KIND_ADJ = 1, KIND_SMEM = 2, KIND_REGADJ = 3, KIND_REGRAG = 4 };
 
 template <int NT, int KIND>
