@@ -185,6 +185,13 @@ __device__ __forceinline__ void pass(cw* z, const ulonglong2* tw, int shift, uns
   }
 }
 
+// the sign bit of a row: multiplicative hashing twice, the high bits folded into the low ones between
+__device__ __forceinline__ unsigned row_sign(unsigned r) {
+  unsigned h = (r + 1u) * 2654435761u;
+  h = (h ^ (h >> 15)) * 2654435761u;
+  return h & 0x80000000u;
+}
+
 // rows 2p, 2p + 1 of w (N doubles each, the first M used) replaced by their transforms times scale.
 // tab: N twiddles ((cos + 1) / 2, (1 - sin) / 2) of angles 2 pi m / N, then s_k, k = 0 .. N / 2 (words)
 template <int N>
@@ -202,15 +209,20 @@ __global__ void __launch_bounds__(N / 16, 512 / (N / 16)) k_dst_fixed(double* w,
 
   // ---------------------------------------------------------------- rows -> words -> y
   // thread t: k = 1 + t + i T and N - k, i = 0..7 (k = N / 2 is its own mirror image)
+  // What bias the products and shifts keep is the same in every row of one scale, and a solve along the
+  // rows' index would add it up over them: each row is negated or not, without a pattern, on its way
+  // in and out.
+  const unsigned neg0 = row_sign(2u * blockIdx.x), neg1 = row_sign(2u * blockIdx.x + 1u);
+  auto flip = [](double a, unsigned g) { return __hiloint2double(__double2hiint(a) ^ (int)g, __double2loint(a)); };
   double a0[8], b0[8], a1[8], b1[8];
   unsigned m0 = 0u, m1 = 0u;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int k = 1 + tid + i * T;
-    a0[i] = r0[k - 1];
-    b0[i] = r0[N - k - 1];
-    a1[i] = r1[k - 1];
-    b1[i] = r1[N - k - 1];
+    a0[i] = flip(r0[k - 1], neg0);
+    b0[i] = flip(r0[N - k - 1], neg0);
+    a1[i] = flip(r1[k - 1], neg1);
+    b1[i] = flip(r1[N - k - 1], neg1);
     m0 = __vimax3_u32(m0, (unsigned)__double2hiint(a0[i]) & 0x7FFFFFFFu, (unsigned)__double2hiint(b0[i]) & 0x7FFFFFFFu);
     m1 = __vimax3_u32(m1, (unsigned)__double2hiint(a1[i]) & 0x7FFFFFFFu, (unsigned)__double2hiint(b1[i]) & 0x7FFFFFFFu);
   }
@@ -340,7 +352,8 @@ __global__ void __launch_bounds__(N / 16, 512 / (N / 16)) k_dst_fixed(double* w,
   const int k0 = units - sc0 - up0, k1 = units - sc1 - up1;
   const int h0 = k0 / 2, h1 = k1 / 2;
   const bool plain = abs(k0) < 900 && abs(k1) < 900;
-  const double f0 = plain ? scale * pow2i(k0) : scale * pow2i(h0), f1 = plain ? scale * pow2i(k1) : scale * pow2i(h1);
+  const double f0 = flip(plain ? scale * pow2i(k0) : scale * pow2i(h0), neg0);
+  const double f1 = flip(plain ? scale * pow2i(k1) : scale * pow2i(h1), neg1);
   const double g0 = pow2i(k0 - h0), g1 = pow2i(k1 - h1);
   double* o0 = reinterpret_cast<double*>(z);
   // X_{2m}, X_{2m+1} of row 0 at o0, of row 1 behind it; one 16-byte slot of padding per 16 pairs
