@@ -1674,7 +1674,12 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     b->n_smem[f] = std::max(b->n_smem[f], q.n);
     if (q.o_fix || b->adj[(size_t)s].rec.o_fix) b->ntf = 1;
   }
-  if (b->ntf) b->ntf = fix_threads(b->NT[FORM_F64], b->n_smem[FORM_F64]);
+  // threads for windows of at most the default rows: one system of longer blocks would double the CTA of
+  // every window (10000 systems of 256 to 2^20 rows, one of 4033 in 65-row blocks: 8.28 ms, so 5.50).  Its
+  // windows are taken as long as their rows fit those threads, in FP64 arithmetic otherwise.
+  if (b->ntf)
+    b->ntf = fix_threads(b->NT[FORM_F64],
+                         o.n_req > 0 ? b->n_smem[FORM_F64] : std::min(b->n_smem[FORM_F64], default_rows(FORM_F64)));
   // MIXED windows take the register path where its shape allows (one-window systems too: 3946 Poisson
   // modes of 4096 rows 80.9 us, on the shared-memory path 93.0), in the kernel that also takes
   // shorter last blocks if such windows are no fewer than the others (600 systems of 5000 rows 30.7 us,

@@ -1012,3 +1012,17 @@ def test_mixed_last_block_of_one_row(D, N, flags):
     ref = oracle.thomas_batched(tm1, t0, tp1, Ns, W.offsets(Ns), Fb)
     assert np.max(np.abs(y - ref)) < TOL * np.max(np.abs(ref))
     assert plan.status() == 0
+
+
+def test_batch_with_blocks_beyond_the_fixed_point_threads(D):
+    """FP64 systems whose lengths ask for other than 64-row blocks (4033: 65 rows in one window; 4033 + 4032 k:
+    neither 64 nor 63 rows) beside full windows, among enough others to keep 64-thread windows."""
+    N = np.array([4033, 4033 + 4032 * 5, 4096, 4097, 70001, 2] + [4096 * 8] * 40)
+    rng = np.random.default_rng(4033)
+    tm1, tp1, t0 = rng.uniform(-1, -0.5, N.size), rng.uniform(-1, -0.5, N.size), rng.uniform(2.05, 4, N.size)
+    F = rng.uniform(-1, 1, int(N.sum()))
+    x, b = batch_solve(D, N, tm1, t0, tp1, F, precision=0)
+    off = W.offsets(N)
+    ref = oracle.thomas_batched(tm1, t0, tp1, N, off, F)
+    for o, n in zip(off, N):
+        assert rel(x[o:o + n], ref[o:o + n]) < TOL
