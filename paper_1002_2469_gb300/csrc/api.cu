@@ -160,18 +160,26 @@ static u64 dd_word(dd v) {
   if (!(f < 0x1p64)) return ~(u64)0;
   return (u64)f + (u64)(long long)std::llround((w - f) + v.l * 0x1p64);
 }
-// x r 2^-64 as the kernels round it
-static u64 word_mul(u64 x, u64 r) {
-  const u64 xh = x >> 32, xl = x & 0xFFFFFFFFu, rh = r >> 32, rl = r & 0xFFFFFFFFu;
-  return xh * rh + ((xl * rh) >> 32) + ((xh * rl) >> 32);
+static dd dd_of(u64 v) { return dd_norm((double)(v >> 32) * 0x1p32, (double)(v & 0xFFFFFFFFu)); }
+static dd dd_frac(u64 w) {
+  const dd v = dd_of(w);
+  return dd{v.h * 0x1p-64, v.l * 0x1p-64};
+}
+// the mean of what fx_mul (fixed.cuh) drops from a product by the word w: about half a unit in each of its
+// two high halves (less the smallest step, which a power of two's product shows), and the product of the
+// low halves
+static double mean_trunc(u64 w) {
+  auto half = [](u64 v) { return v ? 0.5 * (1.0 - 0x1p-32 * (double)(v & (0 - v))) : 0.0; };
+  return half(w >> 32) + half(w & 0xFFFFFFFFu) + 0x1p-33 * (double)(w & 0xFFFFFFFFu);
 }
 
 // The table of one system of N rows; false: its windows are solved in FP64.  Needs both recurrence
 // coefficients of one sign; R^N below 2^-66 (the left end's closed form, window_fix.cuh); the scale g
 // within 2^-60..2^60; and a bound on |X| / max|F| of at most 2^11 (kFixMinBits): the words spend that
 // many bits on the largest possible solution, and the right-hand side keeps at least 52 below its
-// largest value.  Measured rms errors against exact values, FP64 recurrences and words: gain 4 1.2e-16
-// and 5e-17, gain 1000 (tridiag{-1, 2.001, -1}) 4.1e-15 and 2.9e-16.
+// largest value.  Measured rms errors over 2^20 rows of a normal right-hand side, FP64 recurrences and
+// words: tridiag{-1, 4, -1} 1.2e-16 and 4.7e-17, t_0 = 2.05 4.2e-16 and 4.8e-17, t_0 = 2.005 1.7e-15 and
+// 1.0e-16, t_0 = 2.0013 9.9e-16 and 4.3e-16, t_0 = 2.001 2.3e-15 and 8.3e-16.
 constexpr int kFixMinBits = 52;
 static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
   const Roots r = toeplitz_roots(tm1, t0, tp1);
@@ -193,16 +201,16 @@ static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
   T[FX_R] = dd_word(R);
   T[FX_B] = dd_word(B);
   T[FX_G] = dd_word(g);
-  const u64 a = O - word_mul(O, T[FX_B]), K = a - word_mul(a, T[FX_R]);
+  // a = 2^63 (1 - B) and K = a (1 - R) + the mean truncation of the product by R, each to the nearest
+  // unit: a unit's error of K would come out (1 - R)^-1 (1 - B)^-1 times as large, a thousandfold
+  const u64 a = O - ((T[FX_B] >> 1) + (T[FX_B] & 1));
+  const __int128 aR = (__int128)a * T[FX_R] + ((__int128)1 << 63) - (__int128)(mean_trunc(T[FX_R]) * 0x1p64);
+  const u64 K = a - (u64)(int64_t)(aR >> 64);
   int hb = 0;
   while (hb < 63 && (K >> (hb + 1)) != 0) ++hb;
   if (hb < kFixMinBits) return false;
   T[FX_A] = a;
-  T[FX_K] = K + 1;
-  // the mean truncation of the two products per row of Y (settling at 2.5 / (1 - B)), of the last
-  // two products and of the lowest bit set on conversion
-  const double bias = (2.5 / (1.0 - B.h) + 1.25) * g.h + 1.25 - 0.5;
-  T[FX_KG] = (u64)std::llround(bias) - word_mul(O, T[FX_G]);
+  T[FX_K] = K;
   T[FX_HB] = (u64)hb;
   T[FX_GK] = (u64)(int64_t)gk;
   T[FX_FLAGS] = (u64)(((tm1 != 0.0 ? r.rs : r.ib) < 0.0 ? FIX_ALT : 0) | (r.g < 0.0 ? FIX_NEG : 0) |
@@ -227,6 +235,30 @@ static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
     }
     v = dd_mul(v, R);
     w = dd_mul(w, B);
+  }
+  {
+    // The constant of the output product: what the words of a window with F = 0 come to on average, from
+    // the words' own roundings and the products' mean truncations, step by step over the 16 rows of a half
+    // (kernel's steps 1 to 5; its products between halves and threads add the unit that they drop), and
+    // half a unit for the lowest bit set on conversion.
+    const dd one{1.0, 0.0};
+    auto prod = [](u64 w, dd x, double add) { return dd_add(dd_mul(dd_frac(w), x), dd{add - mean_trunc(w), 0.0}); };
+    auto fixpoint = [&](u64 w, dd add) {   // x = x w + add, its product's unit added back
+      const dd f = dd_frac(w);
+      return dd_div(dd_add(add, dd{1.0 - mean_trunc(w), 0.0}), dd_add(one, dd{-f.h, -f.l}));
+    };
+    dd u[kFixHalf];
+    u[0] = dd_of(K);
+    for (int i = 1; i < kFixHalf; ++i) u[i] = dd_add(dd_of(K), prod(T[FX_R], u[i - 1], 0.0));
+    const dd U = fixpoint(T[FX_P + kFixHalf - 1], u[kFixHalf - 1]);
+    for (int i = 0; i < kFixHalf; ++i) u[i] = dd_add(u[i], prod(T[FX_P + i], U, 0.0));
+    for (int i = kFixHalf - 2; i >= 0; --i) u[i] = dd_add(u[i], prod(T[FX_B], u[i + 1], 0.0));
+    const dd X = fixpoint(T[FX_Q], u[0]);
+    dd sum{0.0, 0.0};
+    for (int i = 0; i < kFixHalf; ++i)
+      sum = dd_add(sum, prod(T[FX_G], dd_add(u[i], prod(T[FX_Q + i], X, 0.0)), 0.5));
+    const double m = std::floor(sum.h / kFixHalf), rest = (sum.h - m * kFixHalf + sum.l) / kFixHalf;
+    T[FX_KG] = 0 - ((u64)m + (u64)(int64_t)std::llround(rest));
   }
   // binades from block to block of a window of varying scale: at most half the decay over 32 rows
   {

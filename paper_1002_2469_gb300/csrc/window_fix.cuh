@@ -23,6 +23,9 @@
 //   3. Y over each half from zero: Y_i = W_i + R^(i+1) Uin + B Y_{i+1};
 //   4. Xin, the word beyond each thread, by the mirrored scan (the window's end gets X = 0);
 //   5. x_i = g (Y_i + B^(16-i) Xin - 2^63), converted and scaled by the window's power of two.
+// The products of steps 2 and 4 add back the unit that fx_mul drops on average (a weak system's
+// recurrences would sum it up to hundreds of units); the offset that the rows' products leave is the same
+// everywhere and comes off with the output product's constant (FX_KG, fix_table in api.cu).
 // The right end of the system (x_N = 0) is step 4 itself.  At its left end step 2's u_{-1} = 0 belongs
 // to the system extended to the left with zero right-hand side, whose x_{-1} is g ib X_0; the
 // homogeneous solution that removes it is X_i -= X_0 B R^(i+1) (x_{-1} = 0 exactly, up to
@@ -51,7 +54,7 @@ constexpr int kFixHalf = 16;
 // a plan's fixed-point table (64-bit words, at SysPlan::o_fix): fractions are multiples of 2^-64
 enum FixIdx {
   FX_R = 0, FX_B, FX_G,          // R, B, |g| 2^-gk in [1/2, 1)
-  FX_K, FX_A, FX_KG,             // K (+1: the products' mean truncation), a, constant of the output product
+  FX_K, FX_A, FX_KG,             // K (with the products' mean truncation), a, constant of the output product
   FX_HB, FX_GK, FX_FLAGS,        // hb, gk, FIX_* bits
   FX_LEVR, FX_LEVB,              // scan levels: R^(32 2^lev) (B^...) below 2^-64, at most 5
   FX_STEP,                       // binades neighbouring blocks of a varying window may differ by (0: none)
@@ -94,7 +97,7 @@ __host__ __device__ inline size_t window_fix_smem_bytes(int NTF) {
 
 // s r, s a signed word and r = m 2^-64 2^-x, into a unit 2^(sh - x) times as large (sh >= 0)
 __device__ __forceinline__ u64 fx_move(u64 s, u64 m, int sh) {
-  const long long z = (long long)fx_mul(s ^ (1ull << 63), m, 0ull - (m >> 1));
+  const long long z = (long long)fx_mul(s ^ (1ull << 63), m, 1ull - (m >> 1));
   return (u64)(z >> min(sh, 63));
 }
 // a signed word in a unit 2^sh times as large
@@ -224,12 +227,12 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
   u64 Uin;
   const int levr = (int)fx[FX_LEVR], levb = (int)fx[FX_LEVB];
   if (!var) {
-    u64 E = fx_mul(E1, R16, E2);
-    if (tid == 0) E = fx_mul(a0, tR[1], E);
+    u64 E = fx_mul(E1, R16, E2 + 1);
+    if (tid == 0) E = fx_mul(a0, tR[1], E + 1);
     for (int k = 0; k < levr; ++k) {
       const int d = 1 << k;
       const u64 y = __shfl_up_sync(0xffffffffu, E, d);
-      E = fx_mul(lane < d ? 0ull : y, tR[d], E);
+      E = fx_mul(lane < d ? 0ull : y, tR[d], E + (lane < d ? 0u : 1u));
     }
     if (lane == 31) sw[wid] = E;
     Uin = __shfl_up_sync(0xffffffffu, E, 1);
@@ -239,15 +242,15 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
       u64 C = sw[wid - 1];
       if (levr >= 5) {   // couplings may span several warps
         C = sw[0];
-        for (int w = 1; w < wid; ++w) C = fx_mul(C, tR[32], sw[w]);
+        for (int w = 1; w < wid; ++w) C = fx_mul(C, tR[32], sw[w] + 1);
       }
-      Uin = (lane == 0) ? C : fx_mul(C, tR[lane], Uin);
+      Uin = (lane == 0) ? C : fx_mul(C, tR[lane], Uin + 1);
     } else if (lane == 0) {
       Uin = a0;
     }
   } else {
     // signed words, each in its thread's unit; R <= 2^-1/4 here, so that 16 blocks away nothing is left
-    u64 S = fx_mul(E1, R16, E2) - (a0 - fx_mul(a0, tR[1], 0ull));
+    u64 S = fx_mul(E1, R16, E2 + 1) - (a0 - fx_mul(a0, tR[1], 1ull));
     const int lev = min(4, levr + 1);
     for (int k = 0; k < lev; ++k) {
       const int d = 1 << k;
@@ -269,7 +272,7 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
     Uin = a0 + (lane == 0 ? fx_rescale(C, e - eC) : fx_rescale(y, e - ey));
   }
   // ---------------------------------------------------------------- 3. backward words
-  const u64 Uin2 = fx_mul(Uin, R16, E1);
+  const u64 Uin2 = fx_mul(Uin, R16, E1 + 1);
   u64 Y1 = 0, Y2 = 0;
   {
     const unsigned bh = (unsigned)(fx[FX_B] >> 32), bl = (unsigned)fx[FX_B];
@@ -300,14 +303,14 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
   // ---------------------------------------------------------------- 4. the words beyond the threads
   u64 Xin, E0;   // E0: the thread's first word, complete
   {
-    const u64 loc = fx_mul(Y2, B16, Y1);
+    const u64 loc = fx_mul(Y2, B16, Y1 + 1);
     if (!var) {
       u64 E = (nv == 0) ? 0ull : loc;
-      if (tid == tlast) E = fx_mul(1ull << 63, tB[1], E);
+      if (tid == tlast) E = fx_mul(1ull << 63, tB[1], E + 1);
       for (int k = 0; k < levb; ++k) {
         const int d = 1 << k;
         const u64 y = __shfl_down_sync(0xffffffffu, E, d);
-        E = fx_mul(lane + d > 31 ? 0ull : y, tB[d], E);
+        E = fx_mul(lane + d > 31 ? 0ull : y, tB[d], E + (lane + d > 31 ? 0u : 1u));
       }
       if (lane == 0) sw[NW + wid] = E;
       Xin = __shfl_down_sync(0xffffffffu, E, 1);
@@ -317,12 +320,12 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
         u64 C = sw[NW + wid + 1];
         if (levb >= 5) {
           C = sw[2 * NW - 1];
-          for (int w = NW - 2; w > wid; --w) C = fx_mul(C, tB[32], sw[NW + w]);
+          for (int w = NW - 2; w > wid; --w) C = fx_mul(C, tB[32], sw[NW + w] + 1);
         }
-        Xin = (lane == 31) ? C : fx_mul(C, tB[31 - lane], Xin);
+        Xin = (lane == 31) ? C : fx_mul(C, tB[31 - lane], Xin + 1);
       }
     } else {
-      u64 S = loc - ((1ull << 63) - fx_mul(1ull << 63, tB[1], 0ull));
+      u64 S = loc - ((1ull << 63) - fx_mul(1ull << 63, tB[1], 1ull));
       if (nv == 0) S = 0;
       const int lev = min(4, levb + 1);
       for (int k = 0; k < lev; ++k) {
@@ -345,7 +348,7 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
       Xin = (1ull << 63) + (lane == 31 ? fx_rescale(C, e - eC) : fx_rescale(y, e - ey));
     }
     if (tid >= tlast) Xin = 1ull << 63;
-    E0 = fx_mul(Xin, tB[1], loc);
+    E0 = fx_mul(Xin, tB[1], loc + 1);
   }
   if (flags & FIX_GUARD) {
     // high gain: the words' unit is set by the largest possible |X|; a window whose solution stays far
@@ -394,7 +397,7 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
 
   // ---------------------------------------------------------------- 5. the solution, own rows out
   if (kFixRows * tid < j1 && kFixRows * (tid + 1) > j0) {
-    const u64 X1 = fx_mul(Xin, B16, Y2);
+    const u64 X1 = fx_mul(Xin, B16, Y2 + 1);
     const unsigned xh = (unsigned)(X1 >> 32), xl = (unsigned)X1, yh = (unsigned)(Xin >> 32), yl = (unsigned)Xin;
     const unsigned gh = (unsigned)(fx[FX_G] >> 32), gl = (unsigned)fx[FX_G];
     const u64 kg = fx[FX_KG];
