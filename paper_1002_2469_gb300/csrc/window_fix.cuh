@@ -31,14 +31,19 @@
 // homogeneous solution that removes it is X_i -= X_0 B R^(i+1) (x_{-1} = 0 exactly, up to
 // (R B)^(N - i) R^(i+1) <= R^N, below 2^-64 by fix_table in api.cu).
 //
-// Scale.  A window whose blocks of 32 rows all reach within 2^-4 of its largest |F| has one power of two
-// for all its words (random right-hand sides).  Where |F| varies more but smoothly -- from one block to
-// the next by at most `step` binades, 4 to 8 and at most half the decay of the couplings over a block:
-// the spectra and profiles of smooth sources -- every thread takes the largest exponent of its own and
-// its two neighbours' blocks, and the scans of steps 2 and 4 move signed words between scales.  (What
-// reaches a thread from k + 1 blocks away is then below R^(16 k) of its own range, which the two bits of
-// kFixVarBits cover.)  Anything else (zero stretches, isolated values, Inf and NaN) is solved in FP64,
-// which resolves a solution's tails relative to themselves.
+// Scale.  Words resolve every row to the same absolute unit, FP64 relative to the values around it.  So a
+// window is taken in one power of two for all its words only if no row of its own lies too far below
+// that: the level of a row is the largest |F| of the rows around it, each weakened by the decay of the
+// coupling over their distance (R per row from the left, B from the right; a lower bound of
+// |T^-1| |F| there, which the FP64 recurrences' errors are relative to), and every level has to
+// reach 2^-lv of the power of two (random right-hand sides do; FX_LVL, fix_table in api.cu).
+// A thread sees its own rows and four on both sides (fix_levels).  Where |F| varies more but smoothly -- from one block
+// of 32 rows to the next by at most `step` binades, 4 to 8 and at most half the decay of the couplings over
+// a block: the spectra and profiles of smooth sources -- every thread takes the largest exponent of its own
+// and its two neighbours' blocks, its levels are held to that, and the scans of steps 2 and 4 move signed
+// words between scales.  (What reaches a thread from k + 1 blocks away is then below R^(16 k) <= 2^(-4 k) of
+// its own range: 16/15 into u and again into X, within kFixVarBits.)  Anything else (zero stretches, isolated
+// values, Inf and NaN) is solved in FP64, which resolves a solution's tails relative to themselves.
 //
 // Layout: one 272-byte slot per thread (slots.cuh) (F, W, Y and x in turn, in place); loops
 // unrolled by two row pairs of both halves.
@@ -58,7 +63,8 @@ enum FixIdx {
   FX_HB, FX_GK, FX_FLAGS,        // hb, gk, FIX_* bits
   FX_LEVR, FX_LEVB,              // scan levels: R^(32 2^lev) (B^...) below 2^-64, at most 5
   FX_STEP,                       // binades neighbouring blocks of a varying window may differ by (0: none)
-  FX_P = 12,                     // R^(i+1), i = 0..15
+  FX_DR, FX_DB, FX_LVL,          // decay per row (R, B) and lowest level below the unit, in 1/16 binades
+  FX_P = 16,                     // R^(i+1), i = 0..15
   FX_Q = FX_P + kFixHalf,        // B^(16-i), i = 0..15
   // powers R^(32 t) = m 2^-64 2^-k with m >= 2^63, t = 0..32 (entry 0 unused): the m, then the k, four
   // 16-bit numbers to a word; and B^(32 t)
@@ -71,10 +77,8 @@ enum FixIdx {
 enum FixFlags { FIX_ALT = 1, FIX_NEG = 2, FIX_GUARD = 4 };   // s = -1; g < 0; high gain (step 4's test)
 
 constexpr int kFixSmemWords = 2 * kFixHalf + 2 * 33;   // tables staged in shared memory
-// a window has one scale while none of its blocks of 32 rows lies further below its largest |F|
-constexpr int kFixBlockRange = 4;
 // headroom (bits) of a window of varying scale
-constexpr int kFixVarBits = 2;
+constexpr int kFixVarBits = 1;
 // a high-gain system's window must reach 2^-kFixGuard of the words' bound
 constexpr int kFixGuard = 8;
 
@@ -92,7 +96,7 @@ __host__ __device__ inline int fix_threads(int NT, int n) {
 
 __host__ __device__ inline size_t window_fix_smem_bytes(int NTF) {
   const size_t nw = (size_t)(NTF / 32);
-  return (size_t)NTF * kRegPairBytes + 8 * (size_t)kFixSmemWords + 8 * 3 * nw + 16 + 4 * 2 * nw + 2 * (size_t)NTF;
+  return (size_t)NTF * kRegPairBytes + 8 * (size_t)kFixSmemWords + 8 * 3 * nw + 16 + 8 * 8 * nw + 4 * 2 * nw + 2 * (size_t)NTF;
 }
 
 // s r, s a signed word and r = m 2^-64 2^-x, into a unit 2^(sh - x) times as large (sh >= 0)
@@ -118,6 +122,72 @@ __device__ __forceinline__ double fx_to_f64(u64 z, unsigned ek) {
   return __hiloint2double((int)((unsigned)__double2hiint(d) + ek), __double2loint(d));
 }
 
+// The largest and the lowest level of a thread's rows (nv of them; lowest: of those whose slot it stores), in
+// 1/16 binades: the upper 15 bits of |F|, at most 0.15 binades below the logarithm; dr, db: decays per row,
+// edge: lane 0's four rows before the warp's and lane 31's behind them, the nearest first.  Two rows to
+// a register (i and 16 + i): the chains over both halves in one instruction.
+__device__ __forceinline__ void fix_levels(const unsigned char* mine, int nv, bool own, int dr, int db,
+                                           const double* edge, int lane, int& largest, int& lowest) {
+  constexpr int H = kFixHalf;
+  constexpr unsigned kNone = 0x7FFF7FFFu;
+  unsigned h[H], top = 0u, low = kNone;
+  if (nv == kFixRows) {
+#pragma unroll
+    for (int k = 0; k < H / 2; ++k) {
+      const uint4 v = *reinterpret_cast<const uint4*>(mine + 16 * k);
+      const uint4 w = *reinterpret_cast<const uint4*>(mine + 8 * H + 16 * k);
+      h[2 * k] = __byte_perm(v.y, w.y, 0x7632) & kNone;
+      h[2 * k + 1] = __byte_perm(v.w, w.w, 0x7632) & kNone;
+      top = __vimax3_s16x2(top, h[2 * k], h[2 * k + 1]);
+    }
+  } else {
+    const unsigned* mw = reinterpret_cast<const unsigned*>(mine) + 1;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      h[i] = __byte_perm(i < nv ? mw[2 * i] : 0u, H + i < nv ? mw[2 * (H + i)] : 0u, 0x7632) & kNone;
+      top = __vmaxs2(top, h[i]);
+    }
+  }
+  const unsigned mr = __byte_perm(0u - (unsigned)dr, 0u, 0x1010), mb = __byte_perm(0u - (unsigned)db, 0u, 0x1010);
+  unsigned l = 0u, r = 0u;   // what the last four rows of each half reach to the right, the first four to the left
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    l = __viaddmax_s16x2(l, mr, h[H - 4 + i]);
+    r = __viaddmax_s16x2(r, mb, h[3 - i]);
+  }
+  unsigned pl = __shfl_up_sync(0xffffffffu, l, 1), pr = __shfl_down_sync(0xffffffffu, r, 1);
+  if (lane == 0 || lane == 31) {
+    const unsigned* ew = reinterpret_cast<const unsigned*>(edge + (lane ? 4 : 0)) + 1;
+    const int d = lane ? db : dr;
+    int c = 0;
+#pragma unroll
+    for (int k = 3; k >= 0; --k) c = __viaddmax_s32(c, -d, (int)((ew[2 * k] & 0x7FFFFFFFu) >> 16));
+    if (lane == 0) pl = (unsigned)c << 16;
+    if (lane == 31) pr = (unsigned)c;
+  }
+  l = __byte_perm(pl, l, 0x5432);   // what reaches the halves' first rows from the left
+  r = __byte_perm(r, pr, 0x5432);   // and their last rows from the right
+#pragma unroll
+  for (int i = 0; i < H; ++i) h[i] = l = __viaddmax_s16x2(l, mr, h[i]);
+  if (nv == kFixRows) {
+#pragma unroll
+    for (int i = H - 1; i > 0; i -= 2) {
+      const unsigned u = __viaddmax_s16x2(r, mb, h[i]);
+      r = __viaddmax_s16x2(u, mb, h[i - 1]);
+      low = __vimin3_s16x2(low, u, r);
+    }
+  } else {
+#pragma unroll
+    for (int i = H - 1; i >= 0; --i) {   // (past the last row: no value, no level to keep)
+      const unsigned live = (i < nv ? 0xFFFFu : 0u) | (H + i < nv ? 0xFFFF0000u : 0u);
+      r = __viaddmax_s16x2(r, mb, h[i]) & live;
+      low = __vmins2(low, r | (kNone & ~live));
+    }
+  }
+  largest = max(top & 0xFFFFu, top >> 16);
+  lowest = own ? min(low & 0xFFFFu, low >> 16) : 0x7FFF;
+}
+
 // The window's rows [row_lo, row_lo + len) of a system (own rows [j0, j1) of them), len <= 32 NTF.
 // Returns false, with every thread of the CTA past a barrier and nothing stored, where the window's
 // values do not suit fixed point: the caller then solves it in FP64.
@@ -134,13 +204,21 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
   u64* tB = tR + 33;
   u64* sw = tB + 33;                                         // 3 NW
   u64* sx0 = sw + 3 * NW;                                    // the system's first row (2 entries)
-  unsigned* sexp = reinterpret_cast<unsigned*>(sx0 + 2);     // 2 NW
+  double* sedge = reinterpret_cast<double*>(sx0 + 2);        // 8 NW: rows past the warps' edges
+  int* sexp = reinterpret_cast<int*>(sedge + 8 * NW);        // 2 NW
   short* sblk = reinterpret_cast<short*>(sexp + 2 * NW);     // NTF: exponents of the threads' blocks
   const u64* fx = reinterpret_cast<const u64*>(tab) + pp->o_fix;
   const double* src = A.F + (int64_t)blockIdx.y * A.ldf + pp->off + row_lo;
   double* dst = A.x + (int64_t)blockIdx.y * A.ldx + pp->off + row_lo;
 
   slots_load(smem, src, len, (reinterpret_cast<uintptr_t>(src) & 15u) == 0u, lane, wid);
+  if (lane < 8) {   // four rows on either side of the warp's, the nearest first
+    const int j = lane < 4 ? wid * kWarpRows - 1 - lane : (wid + 1) * kWarpRows + lane - 4;
+    if (j >= 0 && j < len)
+      cp_async8(sedge + 8 * wid + lane, src + j);
+    else
+      sedge[8 * wid + lane] = 0.0;
+  }
   const short* rx = reinterpret_cast<const short*>(fx + FX_RX);
   const short* bx = reinterpret_cast<const short*>(fx + FX_BX);
   for (int i = tid; i < 2 * kFixHalf; i += NTF) tp[i] = fx[FX_P + i];
@@ -153,47 +231,40 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
 
   // ---------------------------------------------------------------- the window's exponent range
   const int nv = max(0, min(kFixRows, len - kFixRows * tid));   // the thread's rows
-  unsigned hmax = 0u, hblk = 0xFFFFFFFFu;
-  if (nv == kFixRows) {
-#pragma unroll
-    for (int k = 0; k < kFixRows / 2; ++k) {
-      const uint4 v = *reinterpret_cast<const uint4*>(mine + 16 * k);
-      hmax = __vimax3_u32(hmax, v.y & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu);
-    }
-    hblk = hmax;
-  } else {
-    for (int i = 0; i < nv; ++i)
-      hmax = max(hmax, reinterpret_cast<const unsigned*>(mine)[2 * i + 1] & 0x7FFFFFFFu);
-  }
-  const int eown = (int)(hmax >> 20);
+  const bool own = kFixRows * tid < j1 && kFixRows * (tid + 1) > j0;   // it stores some of them
+  const int dr = (int)fx[FX_DR], db = (int)fx[FX_DB];
+  int hmax, lvl;   // largest and lowest level of the thread's rows
+  fix_levels(mine, nv, own, dr, db, sedge + 8 * wid, lane, hmax, lvl);
+  const int eown = hmax >> 4;
   sblk[tid] = (short)eown;
   hmax = __reduce_max_sync(0xffffffffu, hmax);
-  hblk = __reduce_min_sync(0xffffffffu, hblk);
+  int lmin = __reduce_min_sync(0xffffffffu, lvl);
   if (lane == 0) {
     sexp[wid] = hmax;
-    sexp[NW + wid] = hblk;
+    sexp[NW + wid] = lmin;
   }
   __syncthreads();
   hmax = sexp[0];
-  hblk = sexp[NW];
+  lmin = sexp[NW];
 #pragma unroll
   for (int w = 1; w < NW; ++w) {
     hmax = max(hmax, sexp[w]);
-    hblk = min(hblk, sexp[NW + w]);
+    lmin = min(lmin, sexp[NW + w]);
   }
-  const int emax = (int)(hmax >> 20), eblk = (int)(hblk >> 20);
+  const int emax = hmax >> 4, lv = (int)fx[FX_LVL];
   const int hb = (int)fx[FX_HB];
   const int tlast = (len - 1) / kFixRows;   // the last thread with rows
   // one scale, |F| 2^sc < 2^hb <= K, for a window of normal finite values with sc >= 0 (zeros convert
   // exactly then); else each thread's own
   if (emax < 192 || emax > 1020 + hb) return false;
-  const bool var = eblk < emax - kFixBlockRange;
+  const bool var = lmin < ((emax + 1) << 4) - lv;
   int e = emax;
   if (var) {
     const int step = (int)fx[FX_STEP];
     const int el = (tid > 0 && nv > 0) ? sblk[tid - 1] : eown, er = (tid < tlast) ? sblk[tid + 1] : eown;
     e = max(eown, max(el, er));
-    const bool ok = nv == 0 || (eown >= 192 && abs(eown - el) <= step && abs(eown - er) <= step);
+    const bool ok = nv == 0 || (eown >= 192 && abs(eown - el) <= step && abs(eown - er) <= step &&
+                                lvl >= ((e + 1 + kFixVarBits) << 4) - lv);
     if (!__syncthreads_and(step > 0 && ok)) return false;
     sblk[tid] = (short)e;   // (read after the next barrier)
   }
@@ -396,7 +467,7 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
   }
 
   // ---------------------------------------------------------------- 5. the solution, own rows out
-  if (kFixRows * tid < j1 && kFixRows * (tid + 1) > j0) {
+  if (own) {
     const u64 X1 = fx_mul(Xin, B16, Y2 + 1);
     const unsigned xh = (unsigned)(X1 >> 32), xl = (unsigned)X1, yh = (unsigned)(Xin >> 32), yl = (unsigned)Xin;
     const unsigned gh = (unsigned)(fx[FX_G] >> 32), gl = (unsigned)fx[FX_G];

@@ -52,3 +52,61 @@ def test_weak_systems_have_no_mean_error(D, t):
     hb = 63 + math.floor(math.log2((1.0 - R) * (1.0 - B)))
     unit = g * 2.0 ** (math.frexp(np.max(np.abs(F)))[1] - hb)
     assert abs(np.mean(s * err)) <= (4.0 / (1.0 - B) + 4.0 + 2.0) * unit
+
+
+def component_bound(t, F):
+    """A priori bound of the FP64 recurrences' errors, row by row: with s, t the two recurrences run on
+    |F| (g t = |T^-1| |F|), constants good to an ulp and their powers to an ulp per row, and 32 roundings of
+    quantities below t for the block ends, the scan and the corrections of the block solves."""
+    R, B, g = roots(t)
+
+    def conv(a, r, order):
+        out, c = np.empty_like(a), np.zeros(a.shape[1:], dtype=a.dtype)
+        for i in order:
+            c = c * r + a[i]
+            out[i] = c
+        return out
+
+    N = F.shape[0]
+    up, down = range(N), range(N - 1, -1, -1)
+    s = conv(np.abs(F).astype(np.longdouble), R, up)
+    y = conv(s, B, down)
+    e = 4.0 * conv(conv(s, R, up), B, down) + 4.0 * conv(y, B, down) + 32.0 * y
+    return g * 2.0 ** -53 * e
+
+
+def sparse(N, rng):
+    """Right-hand sides whose rows differ by many orders of magnitude within a few rows, and ordinary ones."""
+    i = np.arange(N)
+    out = {}
+    out["one value in 32 rows"] = np.where(i % 32 == 7, 1.0 + np.abs(rng.standard_normal(N)), 0.0)
+    out["rows 64 k and 64 k + 63"] = np.where((i % 64 == 0) | (i % 64 == 63), 1.0, 0.0)
+    out["small background"] = np.where(i % 32 == 31, 1.0, 1e-12 * rng.uniform(0.5, 1.0, N))
+    out["large values"] = np.where(i % 32 == 16, 1e10, rng.standard_normal(N))
+    F = rng.standard_normal(N)
+    at = 40
+    while at < N - 100:   # stretches weakened by up to 2^-30
+        n = int(rng.integers(2, 60))
+        F[at:at + n] *= 2.0 ** -rng.uniform(0.0, 30.0)
+        at += n + int(rng.integers(20, 120))
+    out["weak stretches"] = F
+    out["zero stretch at a warp's edge"] = np.where((i % 1024 > 990) | (i % 1024 < 3), 0.0, rng.standard_normal(N))
+    out["sine"] = np.sin(2.0 * np.pi * 5.3 * (i + 0.37) / 4096.0)
+    out["steep"] = rng.uniform(1.0, 2.0, N) * 2.0 ** (-(i % 4096) / 8.0)
+    out["random"] = rng.standard_normal(N)
+    return out
+
+
+@pytest.mark.parametrize("t", [(-1.0, 4.0, -1.0), (-0.5, 8.0, -0.5), (-1.0, 20.0, -1.0), (-1.2, 2.5, -0.8), (1.0, 4.0, 1.0),
+                               (0.7, -2.5, 1.1), (-1.0, 2.05, -1.0), (-1.0, 2.005, -1.0), (0.0, 2.0, -1.0),
+                               (-1.0, 2.0, 0.0)])
+def test_every_row_is_as_good_as_fp64_recurrences_give_it(D, t):
+    N = 4093
+    cases = sparse(N, np.random.default_rng(23))
+    bounds = component_bound(t, np.stack(list(cases.values()), axis=1))
+    # one window, whose block solves leave nothing out
+    plan = D.Plan(*t, N, block_size=64, threads=64, trunc_eps=1e-290)
+    for k, (name, F) in enumerate(cases.items()):
+        x = plan.solve(torch.from_numpy(F).cuda()).cpu().numpy()
+        err, _ = error(x, t, F)
+        assert (np.abs(err) <= bounds[:, k] + 1e-290).all(), (name, float(np.max(np.abs(err) / (bounds[:, k] + 1e-290))))
