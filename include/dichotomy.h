@@ -332,13 +332,12 @@ void dichotomy_batch_destroy(dich_batch_t batch);
 /* ---------------------------------------------------------------- sine transform steps
  * The two steps around the FFT of an orthonormal DST-I of length M along the first axis of an
  * [M][My] array (the Poisson driver's separation of variables, Sec. 3.2), N = M + 1:
- *   dichotomy_dst_pre:  d_a [M][My] -> d_z [ceil(My / 2)][N] complex (interleaved): columns 2p and
- *     2p + 1 as real and imaginary parts of row p; d_coef [N / 2 + 1][2] holds
- *     scale (sin(pi k / N) + 1/2) and scale (sin(pi k / N) - 1/2), scale = sqrt(2 / N) / 2 times
+ *   dichotomy_dst_pre:  d_a [M][My] -> d_z [My][N], one row per column; d_coef [N / 2 + 1][2] holds
+ *     scale (sin(pi k / N) + 1/2) and scale (sin(pi k / N) - 1/2), scale = sqrt(2 / N) times
  *     whatever factor the caller wants on the result;
- *   a forward complex FFT of length N over the rows of d_z;
- *   dichotomy_dst_post: its result d_Z [ceil(My / 2)][N] -> d_X [M][My].
- * d_z, d_Z and d_coef are 16-byte aligned.  Both only enqueue one kernel.
+ *   a forward real FFT of length N over the rows of d_z;
+ *   dichotomy_dst_post: its result d_Z [My][N / 2 + 1] (complex, interleaved) -> d_X [M][My].
+ * d_Z and d_coef are 16-byte aligned.  Both only enqueue one kernel.
  * Errors: DICH_ERR_ARG (sizes below 1, null, misaligned or host pointers), DICH_ERR_UNSUPPORTED (more
  * than 2^31 tiles of 4096 elements), DICH_ERR_CUDA (launch). */
 int dichotomy_dst_pre(int64_t M, int64_t My, const double* d_a, const double* d_coef, double* d_z, void* stream);

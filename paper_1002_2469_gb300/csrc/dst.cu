@@ -3,15 +3,15 @@
 //
 // With N = M + 1 and a_0 = a_N = 0, y_k = sin(pi k / N) (a_k + a_{N-k}) + (a_k - a_{N-k}) / 2 has
 // sum_k y_k exp(-2 pi i k m / N) = C_m - i S_m with X_{2m} = S_m and X_{2m+1} = C_0 / 2 + C_1 + ... + C_m.
-// Two columns j, j + 1 share one complex FFT: z = y(j) + i y(j+1), and
-//   2 C_m(j) = Re Z_m + Re Z_{N-m},  2 S_m(j) = Im Z_{N-m} - Im Z_m,
-//   2 C_m(j+1) = Im Z_m + Im Z_{N-m},  2 S_m(j+1) = Re Z_m - Re Z_{N-m}.
-// The transform's scale sqrt(2 / N) (and the caller's) and these halves are folded into the coefficients
-// c1 = scale (s + 1/2), c2 = scale (s - 1/2) of y_k = c1 a_k + c2 a_{N-k}, y_{N-k} = c2 a_k + c1 a_{N-k}.
+// Every column has a real FFT of its own: two columns in one complex FFT would each carry rounding errors
+// of the larger one's size, and its Inf and NaN.  (cuFFT itself takes two rows at a time at odd lengths above
+// 256.  A Poisson solve of 2000 x 2319 1363 us, with pairs 1299; 1999 x 2319 922 and 765, 3071 x 3071 1565
+// and 1342.)  The transform's scale sqrt(2 / N) (and the caller's) is folded into the coefficients c1 = scale (s + 1/2), c2 = scale (s - 1/2) of y_k = c1 a_k + c2 a_{N-k},
+// y_{N-k} = c2 a_k + c1 a_{N-k}.
 //
 // Each kernel reads and writes its arrays once (the torch expressions they replace made about 15 passes
 // and strided ones among them).  Both move 16 bytes per element; the FP64 pipe (2 operations per clock
-// and SM) bounds them too: 2 operations per element before the FFT, about 2.3 after it.
+// and SM) bounds them too: 2 operations per element before the FFT, about 2 after it.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -22,14 +22,14 @@
 namespace dich {
 
 // ---------------------------------------------------------------- before the FFT
-// a [M][lda] (row k - 1 holds a_k) -> z [ceil(My / 2)][N] (complex).  One CTA: 32 values of k and their
-// mirror images, 64 columns; the tile is transposed in shared memory, so that rows of a are read and
-// rows of z written in runs of 512 bytes.  coef[k] = (c1, c2), k = 0 .. N / 2.
-constexpr int kPreK = 32, kPreJ = 64, kPrePitch = kPreJ + 2;
+// a [M][My] (row k - 1 holds a_k) -> z [My][N].  One CTA: 32 values of k and their
+// mirror images, 64 columns; the tile is transposed in shared memory, so that rows of a are read in runs of
+// 512 bytes and rows of z written in runs of 256.  coef[k] = (c1, c2), k = 0 .. N / 2.
+constexpr int kPreK = 32, kPreJ = 64, kPrePitch = kPreJ + 1;
 
 __global__ void __launch_bounds__(256) k_dst_pre(int64_t M, int64_t My, const double* a, const double2* coef,
-                                                 double2* z) {
-  __shared__ __align__(16) double t1[kPreK * kPrePitch], t2[kPreK * kPrePitch];
+                                                 double* z) {
+  __shared__ double t1[kPreK * kPrePitch], t2[kPreK * kPrePitch];
   const int64_t N = M + 1, tiles_j = (My + kPreJ - 1) / kPreJ;   // one grid dimension: either may be long
   const int64_t k0 = blockIdx.x / tiles_j * kPreK, j0 = blockIdx.x % tiles_j * kPreJ;
   const int64_t half = N / 2;
@@ -50,22 +50,21 @@ __global__ void __launch_bounds__(256) k_dst_pre(int64_t M, int64_t My, const do
     t2[kk * kPrePitch + jj] = v;
   }
   __syncthreads();
-  const int64_t pairs = (My + 1) / 2;
   const int kk = threadIdx.x & 31;
   const int64_t k = k0 + kk;
   if (k > half) return;
 #pragma unroll
-  for (int i = 0; i < kPreJ / 2 / 8; ++i) {
-    const int p = (threadIdx.x >> 5) + 8 * i;
-    if (j0 / 2 + p >= pairs) break;
-    double2* row = z + (j0 / 2 + p) * N;
-    row[k] = *reinterpret_cast<const double2*>(t1 + kk * kPrePitch + 2 * p);
-    if (k >= 1 && 2 * k != N) row[N - k] = *reinterpret_cast<const double2*>(t2 + kk * kPrePitch + 2 * p);
+  for (int i = 0; i < kPreJ / 8; ++i) {
+    const int c = (threadIdx.x >> 5) + 8 * i;
+    if (j0 + c >= My) break;
+    double* row = z + (j0 + c) * N;
+    row[k] = t1[kk * kPrePitch + c];
+    if (k >= 1 && 2 * k != N) row[N - k] = t2[kk * kPrePitch + c];
   }
 }
 
 // ---------------------------------------------------------------- after the FFT
-// Z [ceil(My / 2)][N] -> X [M][My].  One CTA: eight pairs of columns, a warp each, marching over m in
+// Z [My][N / 2 + 1] -> X [M][My].  One CTA: eight pairs of columns, a warp each, marching over m in
 // chunks of 128 (4 per lane) with the running sums carried along; the chunk's 256 rows by 16 columns
 // leave through shared memory in runs of 128 bytes.  The next chunk's values are loaded before the
 // current one is stored.
@@ -76,16 +75,19 @@ __global__ void __launch_bounds__(256) k_dst_post(int64_t M, int64_t My, const d
   const int64_t N = M + 1, pairs = (My + 1) / 2;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t p0 = (int64_t)blockIdx.x * kPostPairs, p = p0 + wid;
-  const double2* z = Z + (p < pairs ? p : 0) * N;
+  const int64_t pitch = N / 2 + 1;
+  const bool two = 2 * p + 1 < My;   // the pair's second column
+  const double2* z0 = Z + (p < pairs ? 2 * p : 0) * pitch;
+  const double2* z1 = z0 + (two ? pitch : 0);
   const int64_t last = M / 2;   // the largest m: X_{2m} up to M, X_{2m+1} up to M
-  double2 q[4], r[4];           // Z_m and Z_{N-m} of the lane's four m
+  double2 q[4], r[4];           // Z_m of both columns, the lane's four m
   auto load = [&](int64_t m0) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int64_t m = m0 + 4 * lane + i;
       const bool in = m <= last && p < pairs;
-      q[i] = in ? __ldcs(z + m) : make_double2(0.0, 0.0);
-      r[i] = (in && m > 0) ? __ldcs(z + (N - m)) : make_double2(0.0, 0.0);   // m = 0: C_0 / 2 = Re Z_0
+      q[i] = in ? __ldcs(z0 + m) : make_double2(0.0, 0.0);
+      r[i] = (in && two) ? __ldcs(z1 + m) : make_double2(0.0, 0.0);
     }
   };
   load(0);
@@ -94,10 +96,14 @@ __global__ void __launch_bounds__(256) k_dst_post(int64_t M, int64_t My, const d
     double c0[4], c1[4], s0[4], s1[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      c0[i] = q[i].x + r[i].x;
-      c1[i] = q[i].y + r[i].y;
-      s0[i] = r[i].y - q[i].y;
-      s1[i] = q[i].x - r[i].x;
+      c0[i] = q[i].x;
+      c1[i] = r[i].x;
+      s0[i] = -q[i].y;
+      s1[i] = -r[i].y;
+    }
+    if (m0 + lane == 0) {   // C_0 / 2
+      c0[0] *= 0.5;
+      c1[0] *= 0.5;
     }
     if (m0 + kPostM <= last) load(m0 + kPostM);
     // inclusive sums over the lane's four, then the exclusive scan of the lanes' totals
@@ -154,11 +160,11 @@ extern "C" {
 
 int dichotomy_dst_pre(int64_t M, int64_t My, const double* d_a, const double* d_coef, double* d_z, void* stream) {
   if (M < 1 || My < 1 || !d_a || !d_coef || !d_z) return DICH_ERR_ARG;
-  if (!aligned8(d_a) || ((uintptr_t)d_coef & 15u) != 0 || ((uintptr_t)d_z & 15u) != 0) return DICH_ERR_ARG;
+  if (!aligned8(d_a) || ((uintptr_t)d_coef & 15u) != 0 || !aligned8(d_z)) return DICH_ERR_ARG;
   if (!is_device_ptr(d_a) || !is_device_ptr(d_coef) || !is_device_ptr(d_z)) return DICH_ERR_ARG;
   const int64_t gk = ((M + 1) / 2 + 1 + kPreK - 1) / kPreK, gj = (My + kPreJ - 1) / kPreJ;
   if (gk > INT32_MAX / gj) return DICH_ERR_UNSUPPORTED;
-  k_dst_pre<<<(unsigned)(gk * gj), 256, 0, (cudaStream_t)stream>>>(M, My, d_a, (const double2*)d_coef, (double2*)d_z);
+  k_dst_pre<<<(unsigned)(gk * gj), 256, 0, (cudaStream_t)stream>>>(M, My, d_a, (const double2*)d_coef, d_z);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? DICH_OK : cuda_fail(e);
 }

@@ -10,8 +10,8 @@ operator; mode k = 1..M leaves one tridiagonal Toeplitz system along y,
 the series of Sec. 3.2 with one t_0 per mode.  All M systems are solved as one batch by the
 Dichotomy kernels (the library's batched entry point); the inverse DST-I (the same transform)
 returns u.  Transforms of length M + 1 = 512 to 4096, a power of two, are the library's own (64-bit fixed
-point on the integer pipes); the others use torch's FFT (cuFFT) of length M + 1 with the library's
-kernels before and after it (two columns per complex row, transposed on the way in and out).
+point on the integer pipes); the others use torch's real FFT (cuFFT) of length M + 1 with the library's
+kernels before and after it (columns transposed to rows on the way in and back on the way out).
 
 Neumann conditions in y (bc_y="neumann"): My cell-centred unknowns y_j = (j + 1/2) / My with
 du/dy = 0 at y = 0 and y = 1 (ghost cells equal to their neighbours).  Mode k then leaves the
@@ -115,7 +115,7 @@ class Poisson2D:
             self._table = torch.from_numpy(words.view(np.int64)).to(dev)
             self._scale = 0.5 * math.sqrt(2.0 / N)
             return
-        c = np.stack([s + 0.5, s - 0.5], axis=1) * (0.5 * math.sqrt(2.0 / N))
+        c = np.stack([s + 0.5, s - 0.5], axis=1) * math.sqrt(2.0 / N)
         dev = self.batch.workspace.device
         self._coef_f = torch.from_numpy(c * (self.hy * self.hy)).to(dev)
         self._coef_v = torch.from_numpy(c).to(dev)
@@ -130,10 +130,10 @@ class Poisson2D:
                                        work.data_ptr(), out.data_ptr(), stream), "dichotomy_dst")
             return out
         coef = self._coef_v if factor == 1.0 else self._coef_f
-        z = torch.empty(((self.My + 1) // 2, self.M + 1), dtype=torch.complex128, device=a.device)
+        z = torch.empty((self.My, self.M + 1), dtype=torch.float64, device=a.device)
         _lib.check(L.dichotomy_dst_pre(self.M, self.My, _d._dev(a, "f"), coef.data_ptr(), z.data_ptr(), stream),
                    "dichotomy_dst_pre")
-        Z = torch.fft.fft(z, dim=-1)
+        Z = torch.fft.rfft(z, dim=-1)
         out = torch.empty_like(a)
         _lib.check(L.dichotomy_dst_post(self.M, self.My, Z.data_ptr(), out.data_ptr(), stream), "dichotomy_dst_post")
         return out
