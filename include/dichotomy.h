@@ -332,16 +332,16 @@ void dichotomy_batch_destroy(dich_batch_t batch);
 /* ---------------------------------------------------------------- sine transform steps
  * The two steps around the FFT of an orthonormal DST-I of length M along the first axis of an
  * [M][My] array (the Poisson driver's separation of variables, Sec. 3.2), N = M + 1:
- *   dichotomy_dst_pre:  d_a [M][My] -> d_z [My][N], one row per column; d_coef [N / 2 + 1][2] holds
+ *   dichotomy_dst_rows_pre:  d_a [M][My] -> d_z [My][N], one row per column; d_coef [N / 2 + 1][2] holds
  *     scale (sin(pi k / N) + 1/2) and scale (sin(pi k / N) - 1/2), scale = sqrt(2 / N) times
  *     whatever factor the caller wants on the result;
  *   a forward real FFT of length N over the rows of d_z;
- *   dichotomy_dst_post: its result d_Z [My][N / 2 + 1] (complex, interleaved) -> d_X [M][My].
+ *   dichotomy_dst_rows_post: its result d_Z [My][N / 2 + 1] (complex, interleaved) -> d_X [M][My].
  * d_Z and d_coef are 16-byte aligned.  Both only enqueue one kernel.
  * Errors: DICH_ERR_ARG (sizes below 1, null, misaligned or host pointers), DICH_ERR_UNSUPPORTED (more
  * than 2^31 tiles of 4096 elements), DICH_ERR_CUDA (launch). */
-int dichotomy_dst_pre(int64_t M, int64_t My, const double* d_a, const double* d_coef, double* d_z, void* stream);
-int dichotomy_dst_post(int64_t M, int64_t My, const double* d_Z, double* d_X, void* stream);
+int dichotomy_dst_rows_pre(int64_t M, int64_t My, const double* d_a, const double* d_coef, double* d_z, void* stream);
+int dichotomy_dst_rows_post(int64_t M, int64_t My, const double* d_Z, double* d_X, void* stream);
 
 /* The whole transform for N = M + 1 = 512, 1024, 2048 or 4096, in 64-bit fixed point on the integer
  * pipes (each column in its own power-of-two unit; results as close to the exact transform as an FP64

@@ -35,7 +35,7 @@ EXPORTS = [
     "dichotomy_batch_destroy", "dichotomy_strerror", "dichotomy_last_cuda_error", "dichotomy_version",
     "dichotomy_gen_plan", "dichotomy_gen_info", "dichotomy_gen_workspace_bytes", "dichotomy_gen_bind",
     "dichotomy_gen_solve", "dichotomy_gen_solve_series", "dichotomy_gen_residual", "dichotomy_gen_status", "dichotomy_gen_destroy",
-    "dichotomy_dst", "dichotomy_dst_pre", "dichotomy_dst_post",
+    "dichotomy_dst", "dichotomy_dst_rows_pre", "dichotomy_dst_rows_post",
     "dichotomy_shard_info", "dichotomy_shard_reduce", "dichotomy_shard_bounds", "dichotomy_shard_finish",
 ]
 
@@ -133,8 +133,8 @@ def load(build_if_missing: bool = True):
             "dichotomy_gen_status": ([P, P, ctypes.POINTER(I)], I),
             "dichotomy_gen_destroy": ([P], None),
             "dichotomy_dst": ([c_int64, c_int64, P, P, c_double, P, P, P], I),
-            "dichotomy_dst_pre": ([c_int64, c_int64, P, P, P, P], I),
-            "dichotomy_dst_post": ([c_int64, c_int64, P, P, P], I),
+            "dichotomy_dst_rows_pre": ([c_int64, c_int64, P, P, P, P], I),
+            "dichotomy_dst_rows_post": ([c_int64, c_int64, P, P, P], I),
             "dichotomy_shard_info": ([P, c_int32, c_int32, ctypes.POINTER(dich_shard_info)], I),
             "dichotomy_shard_reduce": ([P, c_int32, c_int32, P, P, P, c_size_t, ctypes.POINTER(c_double), P], I),
             "dichotomy_shard_bounds": ([P, c_int32, c_int32, ctypes.POINTER(c_double), P, c_size_t,

@@ -158,7 +158,7 @@ using namespace dich::plan;
 
 extern "C" {
 
-int dichotomy_dst_pre(int64_t M, int64_t My, const double* d_a, const double* d_coef, double* d_z, void* stream) {
+int dichotomy_dst_rows_pre(int64_t M, int64_t My, const double* d_a, const double* d_coef, double* d_z, void* stream) {
   if (M < 1 || My < 1 || !d_a || !d_coef || !d_z) return DICH_ERR_ARG;
   if (!aligned8(d_a) || ((uintptr_t)d_coef & 15u) != 0 || !aligned8(d_z)) return DICH_ERR_ARG;
   if (!is_device_ptr(d_a) || !is_device_ptr(d_coef) || !is_device_ptr(d_z)) return DICH_ERR_ARG;
@@ -169,7 +169,7 @@ int dichotomy_dst_pre(int64_t M, int64_t My, const double* d_a, const double* d_
   return e == cudaSuccess ? DICH_OK : cuda_fail(e);
 }
 
-int dichotomy_dst_post(int64_t M, int64_t My, const double* d_Z, double* d_X, void* stream) {
+int dichotomy_dst_rows_post(int64_t M, int64_t My, const double* d_Z, double* d_X, void* stream) {
   if (M < 1 || My < 1 || !d_Z || !d_X) return DICH_ERR_ARG;
   if (!aligned8(d_X) || ((uintptr_t)d_Z & 15u) != 0) return DICH_ERR_ARG;
   if (!is_device_ptr(d_Z) || !is_device_ptr(d_X)) return DICH_ERR_ARG;

@@ -131,11 +131,11 @@ class Poisson2D:
             return out
         coef = self._coef_v if factor == 1.0 else self._coef_f
         z = torch.empty((self.My, self.M + 1), dtype=torch.float64, device=a.device)
-        _lib.check(L.dichotomy_dst_pre(self.M, self.My, _d._dev(a, "f"), coef.data_ptr(), z.data_ptr(), stream),
-                   "dichotomy_dst_pre")
+        _lib.check(L.dichotomy_dst_rows_pre(self.M, self.My, _d._dev(a, "f"), coef.data_ptr(), z.data_ptr(), stream),
+                   "dichotomy_dst_rows_pre")
         Z = torch.fft.rfft(z, dim=-1)
         out = torch.empty_like(a)
-        _lib.check(L.dichotomy_dst_post(self.M, self.My, Z.data_ptr(), out.data_ptr(), stream), "dichotomy_dst_post")
+        _lib.check(L.dichotomy_dst_rows_post(self.M, self.My, Z.data_ptr(), out.data_ptr(), stream), "dichotomy_dst_rows_post")
         return out
 
     def solve(self, f: torch.Tensor) -> torch.Tensor:
