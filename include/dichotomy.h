@@ -111,7 +111,8 @@ typedef struct {
   int32_t halo_l, halo_r;  /* halo blocks per window (0 on the general path) */
   int32_t path;            /* 0 = single window, 1 = halo windows, 2 = general 3-kernel (a weakly
                               dominant FP64-form system of few windows keeps wider halo windows beside
-                              it, which its solves and adjoints of whole device vectors take) */
+                              it, which its solves and adjoints of whole device vectors take; the
+                              intermediates at beta_offset and iface_offset are left all the same) */
   int32_t precision;       /* effective dich_precision (F64 or MIXED) */
   int64_t tiles;           /* CTAs per solve */
   int32_t Lv, Lw;          /* truncated lengths of the block spikes */

@@ -851,8 +851,8 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
     // a window's values do not suit fixed point, such windows take about the general path's time).
     // A system with a window for every SM becomes a plan of such windows; a shorter one stays a plan of
     // the general path (what its shards and its plan information are about) whose solves and adjoints
-    // of whole vectors take these windows too: N = 5894 to 752765 10 to 11 us, on the general path
-    // 78 to 82.
+    // of whole vectors take these windows too, and a short launch after them leaves the general path's
+    // intermediates: N = 5894 to 752765 13 to 14 us, on the general path 78 to 82.
     if (o.NT == 0 && o.n_req == 0 && p->form == FORM_F64 && p->path == PATH_GENERAL &&
         !(o.flags & DICH_FLAG_FORCE_GENERAL)) {
       dich_plan_s q;
@@ -1090,6 +1090,11 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
       w.F = F + k0 * ldf;
       w.x = x + k0 * ldx;
       e = launch(w, (int)std::min<int64_t>(65535, M - k0));
+      if (e != cudaSuccess) return cuda_fail(e);
+    }
+    if (p->path == PATH_GENERAL) {   // a plan of the general path leaves its intermediates all the same
+      e = launch_block_ends(d_plans + sys_offset, d_tabs, p->fwd.rec.P, x + (M - 1) * ldx, (double*)(p->d_ws + p->off_beta),
+                            (double*)(p->d_ws + p->off_iface), st);
       if (e != cudaSuccess) return cuda_fail(e);
     }
   } else if (M > 1) {

@@ -303,6 +303,53 @@ cudaError_t launch_block_scan_batched(const SysPlan* plans, const double* tabs, 
   return cudaGetLastError();
 }
 
+// What the general path leaves per block, from a solution that other windows computed: the first and last
+// values x_s, x_e of eq. 15 / 18 are rows of x, and the block's own ends alpha, omega follow from
+// eq. 7, x_s = alpha + x_{s-1} v_0 + x_{e+1} w_0, x_e = omega + x_{s-1} v_{n-1} + x_{e+1} w_{n-1}; beta is
+// their 2x2 map of eq. 16.  One thread per block; bound by its launch and two
+// dependent loads (a weak solve of 5894 to 200001 rows 10.8 us without it, 13.0 with it; 700001 10.7 and 14.2).
+__global__ void __launch_bounds__(128) k_block_ends(const SysPlan* pp, const double* tabs, const double* x, double* beta,
+                                                    double* iface) {
+  // the next kernel of the stream may begin its launch: it waits for this grid to complete, and this one for
+  // the windows
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int64_t m = (int64_t)blockIdx.x * 128 + threadIdx.x, P = pp->P;
+  const bool in = m < P, last = m == P - 1;
+  // plan and tables are nobody's output: they load while the windows are still being solved
+  const int64_t s = m * pp->n, e = last ? pp->N - 1 : s + pp->n - 1;
+  const double v0 = last ? pp->v0l : pp->v0, w0 = last ? pp->w0l : pp->w0;
+  const double vend = last ? pp->vendl : pp->vend, wend = last ? pp->wendl : pp->wend;
+  int64_t rec = pp->o_bcm;
+  if (in && m < pp->kl)
+    rec = pp->o_bcl + m * kBC;
+  else if (in && m >= P - pp->kr)
+    rec = pp->o_bcr + (m - (P - pp->kr)) * kBC;
+  const double* bc = tabs + pp->tab + rec;
+  const double m00 = bc[BC_M00], m01 = bc[BC_M01], m10 = bc[BC_M10], m11 = bc[BC_M11];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!in) return;
+  const double xs = x[s], xe = x[e], xl = m > 0 ? x[s - 1] : 0.0, xr = last ? 0.0 : x[e + 1];
+  const double alpha = xs - fma(xl, v0, xr * w0), omega = xe - fma(xl, vend, xr * wend);
+  beta[2 * m] = fma(m00, alpha, m01 * omega);
+  beta[2 * m + 1] = fma(m10, alpha, m11 * omega);
+  iface[2 * m] = xs;
+  iface[2 * m + 1] = xe;
+}
+
+cudaError_t launch_block_ends(const SysPlan* plan, const double* tabs, int64_t P, const double* x, double* beta,
+                              double* iface, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((P + 127) / 128));
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_block_ends, plan, tabs, x, beta, iface);
+}
+
 // One CTA per system.  Bound by latency (an FP64 addition is 64 clocks): one pass over the partial sums,
 // two barrier-free reductions in registers and one barrier, launched with programmatic stream
 // serialization like the window kernels.  (505 MIXED windows of one system: the whole adjoint takes

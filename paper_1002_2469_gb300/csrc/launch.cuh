@@ -14,6 +14,10 @@ namespace dich {
 cudaError_t launch_window_f64(int NT, int ntf, int grid, size_t smem, cudaStream_t st, const WinArgs& a, int grid_y = 1);
 cudaError_t launch_window_mixed(int NT, int grid, size_t smem, cudaStream_t st, const WinArgs& a, int grid_y = 1);
 
+// the per-block beta and first/last values that the general path leaves, from a solution x
+cudaError_t launch_block_ends(const SysPlan* plan, const double* tabs, int64_t P, const double* x, double* beta,
+                              double* iface, cudaStream_t st);
+
 // general path: first/last values of every block from per-block beta (global block scan)
 //   beta [2P] -> iface [2P]; scratch needs 6 * ceil(P / kScanChunk) doubles.
 constexpr int kScanThreads = 256;
