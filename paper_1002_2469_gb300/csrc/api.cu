@@ -1190,8 +1190,11 @@ int dichotomy_solve_host(dich_plan_t p, const double* h_F, double* h_x, double* 
   if (overlap(d_F, nb, d_x, nb)) return DICH_ERR_ALIAS;
   if (!is_device_ptr(d_F) || !is_device_ptr(d_x)) return DICH_ERR_ARG;
   const int64_t T = p->tiles;
-  // only independent windows pipeline: the halo path of a plain Toeplitz plan with two or more windows
-  const bool pipe = p->N >= 2 && p->path == PATH_HALO && !p->quasi && T >= 2 && chunks != 1;
+  // only independent windows pipeline: the halo path of a plain Toeplitz plan with two or more windows, but
+  // not the short windows of a system of one default window (pageable memory, N = 4096: whole 41 us,
+  // in 16 pieces 440)
+  const bool one = p->wide.NT != 0 && p->wide.path == PATH_SINGLE;
+  const bool pipe = p->N >= 2 && p->path == PATH_HALO && !one && !p->quasi && T >= 2 && chunks != 1;
   if (!pipe) {
     e = cudaMemcpyAsync(d_F, h_F, nb, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e);
