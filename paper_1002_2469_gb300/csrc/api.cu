@@ -1072,8 +1072,11 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   // plain kernel is the faster one (N = 4000005 20.6 us and 21.4, 32000005 117.0 and 122.7)
   const int ragged = (rec.nlast < rec.n && (wide ? p->wide.tiles : p->tiles) <= kRagWindows) ? 2 : 1;
   a.reg_path = (device_mem && path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? ragged : 0;
-  const int NT = wide ? p->wide.NT : p->NT, ntf = wide ? p->wide.ntf : p->ntf;
-  const size_t smem = smem_bytes(NT, a.n_smem, p->form, ntf);
+  // (nor is the fixed-point form for mapped host memory, nor more than five FP64 windows at a time on an
+  // SM: the link is shared, N = 2^25 1.80 ms, with six windows 1.87, in fixed point 2.58)
+  const int NT = wide ? p->wide.NT : p->NT, ntf = !device_mem ? 0 : wide ? p->wide.ntf : p->ntf;
+  size_t smem = smem_bytes(NT, a.n_smem, p->form, ntf);
+  if (!device_mem && p->form == FORM_F64) smem = std::max<size_t>(smem, 39 * 1024);
   // windows [win0, win0 + grid) of the single and halo paths (all of them unless a range is given)
   const int grid = (int)(wide ? p->wide.tiles : (nwin < 0) ? p->tiles : nwin);
   auto launch = [&](const WinArgs& w, int gy) {

@@ -16,8 +16,9 @@ def D():
     return pkg
 
 
-def enqueued(call, stream):
-    """The nodes (kernels, copies) of what `call` enqueues on `stream`, by stream capture."""
+def enqueued(call, stream, block_of_first=False):
+    """The number of nodes (kernels, copies) that `call` enqueues on `stream`, or the first one's threads per
+    block, by stream capture."""
     cu = ctypes.CDLL("libcuda.so.1")
     h = ctypes.c_void_p(stream.cuda_stream)
     graph, n = ctypes.c_void_p(), ctypes.c_size_t()
@@ -29,8 +30,15 @@ def enqueued(call, stream):
         rc = cu.cuStreamEndCapture(h, ctypes.byref(graph))
     assert rc == 0
     assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    threads = 0
+    if block_of_first:
+        nodes = (ctypes.c_void_p * n.value)()
+        params = (ctypes.c_uint32 * 64)()   # function (8 bytes), grid x y z, block x y z, ...
+        assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+        assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(nodes[0]), params) == 0
+        threads = params[5]
     cu.cuGraphDestroy(graph)
-    return n.value
+    return threads if block_of_first else n.value
 
 
 @pytest.mark.parametrize("N", [600, 3001, 4096])
@@ -51,3 +59,19 @@ def test_short_system_is_copied_whole(D, N):
         s.synchronize()
         assert torch.equal(x, want)
         assert enqueued(call, s) == 3 * pieces
+
+
+@pytest.mark.parametrize("N", [100003, 1 << 20])
+def test_pinned_memory_is_read_by_the_fp64_sweeps(D, N):
+    """FP64-form windows that read and write host memory: one thread per block of the plan's windows (the
+    fixed-point form's blocks of 32 rows each would have more)."""
+    s = torch.cuda.Stream()
+    plan = D.Plan(-1.2, 2.5, -0.8, N, block_size=64, threads=64)
+    F = torch.randn(N, dtype=torch.float64).pin_memory()
+    x = torch.empty(N, dtype=torch.float64, pin_memory=True)
+    call = lambda: D.dichotomy_solve_host(plan.handle, F, x, None, None, 0, s.cuda_stream)  # noqa: E731
+    call()
+    s.synchronize()
+    want = plan.solve(F.cuda()).cpu()
+    assert torch.max(torch.abs(x - want)) <= 1e-13 * torch.max(torch.abs(want))
+    assert enqueued(call, s, block_of_first=True) == 64
