@@ -28,10 +28,10 @@ __global__ void __launch_bounds__(NTF ? NTF : NT, NTF ? 768 / (NTF ? NTF : NT) :
         return;
       __syncthreads();   // every thread is done with the shared memory the FP64 form reuses
     }
-    if (threadIdx.x >= NT) return;   // the barriers below count the first NT threads
   }
   constexpr int NW = NT / 32;
   constexpr int LD = NT + 1;
+  constexpr int LT = NTF ? NTF : NT;              // threads that load (after fixed point declined, all of them)
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int ns = A.n_smem;
   double* S = sm;
@@ -61,8 +61,8 @@ __global__ void __launch_bounds__(NTF ? NTF : NT, NTF ? 768 / (NTF ? NTF : NT) :
     const double* src = (A.mode == MODE_APPLY) ? (A.x + (int64_t)blockIdx.y * A.ldx + off + row_lo)
                                                : (A.F + (int64_t)blockIdx.y * A.ldf + off + row_lo);
     int b = tid / n, i = tid - (tid / n) * n;
-    const int db = NT / n, di = NT - (NT / n) * n;
-    for (int j = tid; j < len; j += NT) {
+    const int db = LT / n, di = LT - (LT / n) * n;
+    for (int j = tid; j < len; j += LT) {
       cp_async8(&S[i * LD + b], src + j);
       i += di;
       b += db;
@@ -73,15 +73,16 @@ __global__ void __launch_bounds__(NTF ? NTF : NT, NTF ? 768 / (NTF ? NTF : NT) :
     }
   }
   // tables -> smem (overlaps the copies in flight)
-  for (int i = tid; i < Lv; i += NT) tv[i] = tab[pp->o_v + i];
-  for (int i = tid; i < Lw; i += NT) tw[i] = tab[pp->o_w + i];
+  for (int i = tid; i < Lv; i += LT) tv[i] = tab[pp->o_v + i];
+  for (int i = tid; i < Lw; i += LT) tw[i] = tab[pp->o_w + i];
   if (has_last)
-    for (int i = tid; i < nlast; i += NT) {
+    for (int i = tid; i < nlast; i += LT) {
       tvl[i] = tab[pp->o_vl + i];
       twl[i] = tab[pp->o_wl + i];
     }
   cp_async_wait_all();
-  sync_first<NT, NTF ? NTF : NT>();
+  __syncthreads();
+  if (LT > NT && threadIdx.x >= NT) return;   // the barriers below count the first NT threads
 
   // ---------------------------------------------------------------- local sweeps (a1)
   const bool act = tid < nwin;

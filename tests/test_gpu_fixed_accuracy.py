@@ -110,3 +110,20 @@ def test_every_row_is_as_good_as_fp64_recurrences_give_it(D, t):
         x = plan.solve(torch.from_numpy(F).cuda()).cpu().numpy()
         err, _ = error(x, t, F)
         assert (np.abs(err) <= bounds[:, k] + 1e-290).all(), (name, float(np.max(np.abs(err) / (bounds[:, k] + 1e-290))))
+
+
+@pytest.mark.parametrize("N", [4096, 100003])
+def test_zero_and_subnormal_windows(D, N):
+    """Windows of zeros have the zero solution; values near the lower end of the FP64 range (whose upper bits
+    are those of zero too) are solved: spacing 2^-1074, at most a few roundings of it."""
+    t = (-1.0, 4.0, -1.0)
+    plan = D.Plan(*t, N, block_size=64, threads=64)
+    x = plan.solve(torch.zeros(N, dtype=torch.float64, device="cuda"))
+    assert (x == 0.0).all()
+    F = np.zeros(N)
+    F[N // 2:N // 2 + 40] = 1000.0 * 2.0 ** -1074
+    F[N // 3] = -3e-310
+    x = plan.solve(torch.from_numpy(F).cuda()).cpu().numpy()
+    ref = oracle.thomas(t, F * 2.0 ** 600) * 2.0 ** -600
+    assert np.max(np.abs(x - ref)) <= 16 * 2.0 ** -1074
+    assert np.max(np.abs(x)) > 1e-311
