@@ -442,13 +442,15 @@ int build_system(double tm1, double t0, double tp1, int64_t N, int NT, int form,
   p.o_klf = take(kl * 4);
   p.o_krf = take(kr * 4);
   p.o_midf = take(66);
-  // the fixed-point table of FP64-form systems (left out where the caller's storage has no room for it)
+  // the fixed-point table of FP64-form systems, 16-byte aligned within the tables (left out on the general
+  // path, which does not use it, and where the caller's storage has no room for it)
   u64 fix[FX_WORDS] = {};
-  const bool with_fix = form == FORM_F64 && fix_threads(NT, n) != 0 && fix_table(tm1, t0, tp1, N, fix) &&
-                        (!sb.ext || (size_t)o_ + FX_WORDS <= sb.ext_cap);
+  const int64_t o_even = o_ + (o_ & 1);
+  const bool with_fix = form == FORM_F64 && sb.path != PATH_GENERAL && fix_threads(NT, n) != 0 &&
+                        fix_table(tm1, t0, tp1, N, fix) && (!sb.ext || (size_t)o_even + FX_WORDS <= sb.ext_cap);
   p.o_fix = 0;
   if (with_fix) {
-    o_ += o_ & 1;   // 16-byte aligned within the table
+    o_ = o_even;
     p.o_fix = take(FX_WORDS);
   }
   // warp-scan levels of the MIXED tree: a contribution from 2^(lev+1) or more blocks away carries a
