@@ -122,6 +122,20 @@ void split_ff(double d, float& h, float& l) {
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// SMs of the current device (0 when no device is visible: plans are then built for the defaults)
+int device_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return sms;
+}
+
 // ---------------------------------------------------------------- fixed-point tables (window_fix.cuh)
 // double-double arithmetic: the fractions carry 64 bits
 struct dd {
@@ -648,6 +662,7 @@ struct dich_plan_s {
   int path = PATH_SINGLE;
   int n_smem = 2;
   int ntf = 0;                         // fixed-point threads of the FP64 form's launches (0: none)
+  int sms = 0;                         // of the device it is bound on
   int64_t tiles = 0;
   SysBuild fwd, adj;
   // the default geometry of a plan that took a latency-bound one: many right-hand sides of a series
@@ -793,20 +808,6 @@ static int plan_geometry(dich_plan_s* p, const Opts& o, int NT, int n) {
                ? fix_threads(NT, n)
                : 0;
   return DICH_OK;
-}
-
-// SMs of the current device (0 when no device is visible: plans are then built for the defaults)
-static int device_sms() {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return sms;
 }
 
 int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich_opts* opts, dich_plan_t* out) {
@@ -1024,6 +1025,7 @@ int dichotomy_plan_bind(dich_plan_t p, void* d_ws, size_t bytes, void* stream) {
   if (e != cudaSuccess) return cuda_fail(e);
   p->d_ws = (char*)d_ws;
   p->d_ws_bytes = bytes;
+  p->sms = device_sms();
   return DICH_OK;
 }
 
@@ -1068,11 +1070,15 @@ static int plan_launch(dich_plan_t p, const double* F, double* x, const double* 
   a.ldx = ldx;
   // the register path only for full solves of device memory, unless the plan asks
   // for the shared-memory path (the general path's passes always take that one).  A shorter last block
-  // puts the last window on that path, which takes longer than the others: launches whose windows
-  // all run at once take the kernel that has such blocks on the register path too (N = 752765 10.1 us,
-  // without it 14.9); with more windows it hides behind the others, as the first to start, and the
-  // plain kernel is the faster one (N = 4000005 20.6 us and 21.4, 32000005 117.0 and 122.7)
-  const int ragged = (rec.nlast < rec.n && (wide ? p->wide.tiles : p->tiles) <= kRagWindows) ? 2 : 1;
+  // puts the last window on that path, which takes longer than the others: systems whose windows
+  // all run at once take the kernel that has such blocks on the register path too (128 threads, 912
+  // windows on 152 SMs: 900 of them 17.6 us, without it 19.8; 64 threads 1500 16.8 and 18.5; 256 threads
+  // 450 18.9 and 22.1); with more windows it hides behind the others, as the first to start, and the
+  // plain kernel is the faster one (930 of 128 threads 20.1 us and 20.9, 32000005 rows 117.0 and 122.7;
+  // 64 threads, 1672 at once, 1824 19.7 and 20.4; 256 threads 600 24.2 and 24.7).  In a series every right-hand side has such
+  // a window: there the windows of one count (1024 x 20011 rows 127.7 us, without it 147.2)
+  const int ragged = (rec.nlast < rec.n && (wide ? p->wide.tiles : p->tiles) <=
+                      windows_at_once(wide ? p->wide.NT : p->NT, a.n_smem, p->sms)) ? 2 : 1;
   a.reg_path = (device_mem && path != PATH_GENERAL && !(p->opts.flags & DICH_FLAG_SMEM_PATH)) ? ragged : 0;
   // (nor is the fixed-point form for mapped host memory, nor more than five FP64 windows at a time on an
   // SM: the link is shared, N = 2^25 1.80 ms, with six windows 1.87, in fixed point 2.58)

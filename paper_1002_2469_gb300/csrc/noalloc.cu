@@ -138,7 +138,7 @@ extern "C" int dichotomy_solve_noalloc(double t_m1, double t_0, double t_1, int6
   a.mode = MODE_FULL;
   a.n_smem = n;
   const int64_t tiles = ceil_div(sb.rec.P, sb.rec.own);
-  a.reg_path = (sb.rec.nlast < n && tiles <= kRagWindows) ? 2 : 1;   // as a plan's; F and x are device memory (checked above)
+  a.reg_path = (sb.rec.nlast < n && tiles <= windows_at_once(NT, n, device_sms())) ? 2 : 1;   // as a plan's; F and x are device memory (checked above)
   const int ntf = (form == FORM_F64 && sb.path != PATH_GENERAL && sb.rec.o_fix) ? fix_threads(NT, n) : 0;
   const size_t smem = smem_bytes(NT, n, form, ntf);
   auto launch = [&](const WinArgs& w) {

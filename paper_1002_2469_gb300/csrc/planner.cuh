@@ -1,6 +1,7 @@
 // planner.cuh -- host-side planning internals shared by the C-ABI translation units
 // (C++ linkage, not exported).  Definitions live in api.cu.
 #pragma once
+#include <algorithm>
 #include <cstddef>
 #include <cstdint>
 #include <string>
@@ -13,7 +14,6 @@ namespace dich {
 namespace plan {
 
 constexpr size_t kAlign = 256;
-constexpr int64_t kRagWindows = 768;   // MIXED windows that run at once (five CTAs on each SM)
 // shared-memory budget per CTA for library-chosen block sizes (several CTAs share an SM so
 // the load, sweeps, tree and store of different windows overlap)
 constexpr size_t kSmemBudget = 110 * 1024;
@@ -53,6 +53,13 @@ size_t smem_bytes(int NT, int n, int form, int ntf = 0);
 int max_rows(int NT, int form, size_t budget);
 int default_threads(int form);
 int default_rows(int form);
+int device_sms();
+// MIXED windows of NT threads and n rows a block that run at once: the forward kernels are built for 768
+// threads on an SM, and its 228 KB of shared memory hold a window's (and 1 KB a CTA) so many times
+inline int64_t windows_at_once(int NT, int n, int sms) {
+  const int64_t fit = (228 * 1024) / (int64_t)(smem_bytes(NT, n, FORM_MIXED) + 1024);
+  return sms * std::min<int64_t>(768 / NT, fit);
+}
 int validate_t(double tm1, double t0, double tp1, int flags = 0);
 int read_opts(const dich_opts* o, Opts& out);
 int pick_form(int prec, const Roots& r);
