@@ -26,7 +26,8 @@
  *
  * The method (what each call computes)
  *   N rows are split into P blocks of n rows (the last block takes the remainder; every
- *   block has >= 2 rows, Sec. 2.1).  The Toeplitz preliminary calculation (Sec. 3.1,
+ *   block has >= 2 rows, Sec. 2.1, but for MIXED systems of 16 k + 1 rows, whose library-chosen
+ *   blocks of 16 rows leave one row to the last).  The Toeplitz preliminary calculation (Sec. 3.1,
  *   Theorem 1 / eq. 20, in the exact factored form of eq. 24-25) is done once per
  *   (t, n): recurrence roots, the two boundary spikes of the block operator T_n and the
  *   O(1) per-block exterior ratios Z (eq. 10-12).  A solve then (a) sweeps every block
@@ -106,7 +107,7 @@ typedef struct {
 /* Read-only description of a plan (for tests, tuning and reporting). */
 typedef struct {
   int64_t N, P;            /* rows, blocks */
-  int32_t n, n_last;       /* block size, size of the last block */
+  int32_t n, n_last;       /* block size, size of the last block (1 only in the MIXED form) */
   int32_t threads;         /* CTA width (window blocks) */
   int32_t halo_l, halo_r;  /* halo blocks per window (0 on the general path) */
   int32_t path;            /* 0 = single window, 1 = halo windows, 2 = general 3-kernel (a weakly
