@@ -87,9 +87,11 @@ constexpr int kFixGuard = 8;
 
 // threads of a CTA that tries the fixed-point form on windows of NT blocks of n rows: 32 rows per thread
 // in one of the compiled widths (at least NT, which the FP64 form needs), 0 where it is not used.
-// Blocks shorter than 32 rows are the planner's (or the caller's) choice for systems that cannot fill
-// the chip, where the sweeps' latency counts: there the FP64 sweeps over short blocks are the shorter
-// chain (113 systems of 4096 rows beside 3983 MIXED ones: 104.7 us for the batch, 106.2 with this form).
+// It is used where the window's rows, 32 to a thread, need at least NT threads: blocks of 16 rows and more in
+// 64-thread windows, of more than 16 in 128- and 256-thread ones.  Shorter blocks are the planner's (or the
+// caller's) choice for systems that cannot fill the chip, where the sweeps' latency counts: there the FP64
+// sweeps over them are the shorter chain (113 systems of 4096 rows in 256-thread windows of 16-row blocks,
+// beside 3983 MIXED ones: 104.7 us for the batch, 106.2 with this form).
 // Windows longer than 8192 rows would exceed 256 threads.
 __host__ __device__ inline int fix_threads(int NT, int n) {
   const int64_t rows = (int64_t)NT * n;

@@ -127,3 +127,25 @@ def test_zero_and_subnormal_windows(D, N):
     ref = oracle.thomas(t, F * 2.0 ** 600) * 2.0 ** -600
     assert np.max(np.abs(x - ref)) <= 16 * 2.0 ** -1074
     assert np.max(np.abs(x)) > 1e-311
+
+
+@pytest.mark.parametrize("t", [(-1.0, 4.0, -1.0), (-1.2, 2.5, -0.8), (1.0, 4.0, 1.0), (0.7, -2.5, 1.1)])
+@pytest.mark.parametrize("N", [1984, 3001, 4031, 4096, 100005])
+def test_rows_of_varying_scale(D, t, N):
+    """A right-hand side that falls by 9 to 20 decades from block to block (windows whose threads each have
+    their own unit), a slope with sign changes and one with a noisy tail: every row against the bound of the
+    values around it, so a wrong unit in the tail shows.  Halos truncate at 2^-64 of values at most 2^8
+    times the row's own, far below the bound."""
+    rng = np.random.default_rng(N)
+    i = np.arange(N)
+    m = np.minimum(i % 4096, 4096 - i % 4096) / 4096.0
+    cases = {"gaussian": rng.uniform(1.0, 2.0, N) * np.exp(-46.0 * (i / N - 0.4) ** 2 / 0.36),
+             "triangle": rng.uniform(1.0, 2.0, N) * 2.0 ** (-100.0 * m),
+             "signs": np.sin(0.013 * i + 0.1) * 2.0 ** (-60.0 * m)}
+    bounds = component_bound(t, np.stack(list(cases.values()), axis=1))
+    n = -(-N // 64)
+    plan = D.Plan(*t, N, block_size=n + (N % n == 1), threads=64) if N <= 4096 else D.Plan(*t, N, block_size=64, threads=64)
+    for k, (name, F) in enumerate(cases.items()):
+        x = plan.solve(torch.from_numpy(F).cuda()).cpu().numpy()
+        err, _ = error(x, t, F)
+        assert (np.abs(err) <= bounds[:, k]).all(), (name, float(np.max(np.abs(err) / bounds[:, k])))
