@@ -220,8 +220,11 @@ static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
   const u64 a = O - ((T[FX_B] >> 1) + (T[FX_B] & 1));
   const __int128 aR = (__int128)a * T[FX_R] + ((__int128)1 << 63) - (__int128)(mean_trunc(T[FX_R]) * 0x1p64);
   const u64 K = a - (u64)(int64_t)(aR >> 64);
+  // |F| < 2^hb <= a (1 - R): the largest FP64 value below 2^hb leaves K's mean truncation room, but for the
+  // few last bits of the smallest hb
+  const u64 room = K >> 57 ? K : K - 3;
   int hb = 0;
-  while (hb < 63 && (K >> (hb + 1)) != 0) ++hb;
+  while (hb < 63 && (room >> (hb + 1)) != 0) ++hb;
   if (hb < kFixMinBits) return false;
   T[FX_A] = a;
   T[FX_K] = K;
