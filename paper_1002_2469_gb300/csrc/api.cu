@@ -282,20 +282,22 @@ static bool fix_table(double tm1, double t0, double tp1, int64_t N, u64* T) {
     double st = 8.0;
     if (R.h > 0.0) st = std::min(st, std::floor(-16.0 * std::log2(R.h)));
     if (B.h > 0.0) st = std::min(st, std::floor(-16.0 * std::log2(B.h)));
-    T[FX_STEP] = (st >= 4.0 && hb - kFixVarBits >= kFixMinBits) ? (u64)st : 0;
+    const int spare = std::ldexp((double)K, -hb) >= 1.14 ? 0 : 1;   // (16/15)^2, window_fix.cuh
+    T[FX_SPARE] = (u64)spare;
+    T[FX_STEP] = (st >= 4.0 && hb - spare >= kFixMinBits) ? (u64)st : 0;
   }
-  // Lowest level of a window's rows below its power of two (window_fix.cuh): hb - 53 binades, what the level
+  // Lowest level of a window's rows below its power of two (window_fix.cuh): hb - 52.5 binades, what the level
   // leaves out of |T^-1| |F| (1 / (1 - R B)) and up to half a binade that the FP64 recurrences' longer sums
   // of errors give, but not below 4 (where couplings reach over hundreds of rows, which a level does not
-  // see).  There the words' errors, relative to |T^-1| |F|, are those of the FP64 recurrences, in all other
-  // rows they are smaller (rms 1.07 and 1.10 times 2^-53 for tridiag{-1, 4, -1} at 9.4 binades, 0.24 and
-  // 0.61 at 5; {-1.2, 2.5, -0.8} 1.13 and 1.21 at 8).  Of windows of 4096 normal values it refuses fewer
-  // than 0.1% at R = 0.27 and above, 0.5% at 0.17, 4% at 0.13 and half of them at 0.05.
+  // see).  Measured errors relative to |T^-1| |F| in windows with rows within 0.3 binades of that level, a
+  // window's largest one in words over the FP64 recurrences': median 0.46 to 1.1 over systems of R = 0.02 to
+  // 0.6, 0.1 to 0.4 of 0.7 to 0.97; rms over the window 0.1 to 0.9.  Of windows of 4096 normal values it refuses
+  // fewer than 0.1% at R = 0.27 and above, 2% at 0.13 and 20% at 0.05.
   auto decay = [](double v) { return (u64)(v > 0.0 ? std::min(std::ceil(-16.0 * std::log2(v)), 0x1p14) : 0x1p14); };
   T[FX_DR] = decay(R.h);
   T[FX_DB] = decay(B.h);
   const double gain = -std::log2(1.0 - R.h * B.h), sums = -0.5 * std::log2((1.0 - R.h) * (1.0 - B.h));
-  T[FX_LVL] = (u64)std::ceil(16.0 * std::max(4.0, hb - 53.0 + gain + std::min(0.5, sums)));
+  T[FX_LVL] = (u64)std::ceil(16.0 * std::max(4.0, hb - 52.5 + gain + std::min(0.5, sums)));
   auto powers = [&](dd r, int at_m, int at_x) {
     dd p = r;
     for (int t = 1; t <= 32; ++t) {

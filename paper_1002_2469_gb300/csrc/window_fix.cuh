@@ -37,12 +37,13 @@
 // coupling over their distance (R per row from the left, B from the right; a lower bound of
 // |T^-1| |F| there, which the FP64 recurrences' errors are relative to), and every level has to
 // reach 2^-lv of the power of two (random right-hand sides do; FX_LVL, fix_table in api.cu).
-// A thread sees its own rows and four on both sides (fix_levels).  Where |F| varies more but smoothly -- from one block
-// of 32 rows to the next by at most `step` binades, 4 to 8 and at most half the decay of the couplings over
+// A thread sees its own rows and four on both sides (fix_levels).  Where |F| varies more but smoothly -- from one
+// block of 32 rows to the next by at most `step` binades, 4 to 8 and at most half the decay of the couplings over
 // a block: the spectra and profiles of smooth sources -- every thread takes the largest exponent of its own
-// and its two neighbours' blocks, its levels are held to that, and the scans of steps 2 and 4 move signed
+// and its two neighbours' blocks, its levels are held to that (and its unit to kFixSlope binades from the
+// next thread's), and the scans of steps 2 and 4 move signed
 // words between scales.  (What reaches a thread from k + 1 blocks away is then below R^(16 k) <= 2^(-4 k) of
-// its own range: 16/15 into u and again into X, within kFixVarBits.)  Anything else (zero stretches, isolated
+// its own range: 16/15 into u and again into X, for which K has room or a bit is kept, FX_SPARE.)  Anything else (zero stretches, isolated
 // values, Inf and NaN) is solved in FP64, which resolves a solution's tails relative to themselves.
 // (Such a window pays for the copy and the test on top: 33554467 rows with a zero stretch in every window 456 us,
 // in FP64 windows alone 441; 1000003 rows, fewer than two windows an SM, 21.9 and 19.6.)  A window of zeros is its
@@ -67,6 +68,7 @@ enum FixIdx {
   FX_LEVR, FX_LEVB,              // scan levels: R^(32 2^lev) (B^...) below 2^-64, at most 5
   FX_STEP,                       // binades neighbouring blocks of a varying window may differ by (0: none)
   FX_DR, FX_DB, FX_LVL,          // decay per row (R, B) and lowest level below the unit, in 1/16 binades
+  FX_SPARE,                      // headroom (bits, 0 or 1) of a window of varying scale
   FX_P = 16,                     // R^(i+1), i = 0..15
   FX_Q = FX_P + kFixHalf,        // B^(16-i), i = 0..15
   // powers R^(32 t) = m 2^-64 2^-k with m >= 2^63, t = 0..32 (entry 0 unused): the m, then the k, four
@@ -80,8 +82,9 @@ enum FixIdx {
 enum FixFlags { FIX_ALT = 1, FIX_NEG = 2, FIX_GUARD = 4 };   // s = -1; g < 0; high gain (step 4's test)
 
 constexpr int kFixSmemWords = 2 * kFixHalf + 2 * 33;   // tables staged in shared memory
-// headroom (bits) of a window of varying scale
-constexpr int kFixVarBits = 1;
+// binades from a thread's unit to the next in a window of varying scale: the words that come from the next
+// thread have its unit's errors
+constexpr int kFixSlope = 2;
 // a high-gain system's window must reach 2^-kFixGuard of the words' bound
 constexpr int kFixGuard = 8;
 
@@ -256,7 +259,7 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
     hmax = max(hmax, sexp[w]);
     lmin = min(lmin, sexp[NW + w]);
   }
-  const int emax = hmax >> 4, lv = (int)fx[FX_LVL];
+  const int emax = hmax >> 4, lv = (int)fx[FX_LVL], spare = (int)fx[FX_SPARE];
   const int hb = (int)fx[FX_HB];
   const int tlast = (len - 1) / kFixRows;   // the last thread with rows
   if (hmax == 0 && A.xf == nullptr) {   // nothing but zeros (or values near the lower end of the FP64 range)?
@@ -278,13 +281,14 @@ __device__ __forceinline__ bool window_fix(const WinArgs& A, const SysPlan* pp, 
   if (var) {
     const int step = (int)fx[FX_STEP];
     const int el = (tid > 0 && nv > 0) ? sblk[tid - 1] : eown, er = (tid < tlast) ? sblk[tid + 1] : eown;
+    const int ell = (tid > 1 && nv > 0) ? sblk[tid - 2] : el, err = (tid + 1 < tlast) ? sblk[tid + 2] : er;
     e = max(eown, max(el, er));
     const bool ok = nv == 0 || (eown >= 192 && abs(eown - el) <= step && abs(eown - er) <= step &&
-                                lvl >= ((e + 1 + kFixVarBits) << 4) - lv);
+                                max(ell, err) <= e + kFixSlope && lvl >= ((e + 1 + spare) << 4) - lv);
     if (!__syncthreads_and(step > 0 && ok)) return false;
     sblk[tid] = (short)e;   // (read after the next barrier)
   }
-  const int sc = hb - (e - 1022) - (var ? kFixVarBits : 0);
+  const int sc = hb - (e - 1022) - (var ? spare : 0);
   const u64 K = fx[FX_K], a0 = fx[FX_A];
   const unsigned flags = (unsigned)fx[FX_FLAGS];
   const unsigned alt = (flags & FIX_ALT) ? 0x80000000u : 0u;
