@@ -335,7 +335,8 @@ def run_gpu(args):
         torch.cuda.empty_cache()
         only = None if args.only is None else set(args.only.split(","))
         others = other_configs(D, W, oracle, stream, world, steps=max(5, min(args.steps, 20)), only=only,
-                               cpu_leg=(rank == 0 and not args.no_cpu_baseline), c4_systems=args.c4_systems)
+                               cpu_leg=(rank == 0 and not args.no_cpu_baseline), c4_systems=args.c4_systems,
+                               poisson_m=args.poisson_m)
 
     if rank != 0:
         return
@@ -497,7 +498,7 @@ def cusparse_comparator(W, oracle, stream, steps):
 OTHER_CONFIGS = ("cusparse", "c1", "c2w", "c3", "c4", "c5", "f3", "f3n", "f4", "table1")
 
 
-def other_configs(D, W, oracle, stream, world, steps=10, only=None, cpu_leg=True, c4_systems=0):
+def other_configs(D, W, oracle, stream, world, steps=10, only=None, cpu_leg=True, c4_systems=0, poisson_m=4095):
     """C1 (latency), the weakly dominant C2 variant, C3 (2-D Poisson modes), C4 (uneven series),
     C5 (adjoint), the rows beyond the hot path and the paper's Table 1 run: time and Gunknowns/s
     per form, with the error against the oracle (on a sample of systems for the batches).
@@ -678,7 +679,7 @@ def other_configs(D, W, oracle, stream, world, steps=10, only=None, cpu_leg=True
         # batched Dichotomy solve, inverse DST-I; manufactured solution u* ~ U[-1, 1]
         from paper_1002_2469_gb300 import poisson as PS
         from oracle import poisson as OP
-        M = 4095
+        M = poisson_m
         us = np.random.default_rng(0).uniform(-1.0, 1.0, (M, M))
         fd = torch.from_numpy(OP.laplacian5(us)).cuda()
         solver = PS.Poisson2D(M)
@@ -687,9 +688,10 @@ def other_configs(D, W, oracle, stream, world, steps=10, only=None, cpu_leg=True
         v = torch.empty_like(rhs)
         ms_solve = _time_batch(lambda: solver.batch.solve(rhs, out=v), steps, world, stream)
         u = solver.solve(fd).cpu().numpy()
-        out["f3_poisson2d_4095"] = {"unknowns": M * M, "ms_total": round(ms_total, 4), "ms_dichotomy": round(ms_solve, 4),
+        transform = "FFT in 64-bit fixed point" if M + 1 in (512, 1024, 2048, 4096) else "FFT by cuFFT"
+        out["f3_poisson2d_%d" % M] = {"unknowns": M * M, "ms_total": round(ms_total, 4), "ms_dichotomy": round(ms_solve, 4),
                                     "Gunknowns_s": round(M * M / ms_total / 1e6, 2),
-                                    "form": "AUTO per mode", "transform": "DST-I, FFT in 64-bit fixed point",
+                                    "form": "AUTO per mode", "transform": "DST-I, " + transform,
                                     "rel_err_vs_manufactured": float(np.max(np.abs(u - us)) / np.max(np.abs(us)))}
         del fd, rhs, v, solver
         torch.cuda.empty_cache()
@@ -843,6 +845,8 @@ def main():
     ap.add_argument("--no-other-configs", action="store_true")
     ap.add_argument("--c4-systems", type=int, default=0,
                     help="time only the first K systems of the uneven series (a smaller case for profiling)")
+    ap.add_argument("--poisson-m", type=int, default=4095,
+                    help="grid points per direction of the Poisson driver (another transform length, for profiling)")
     ap.add_argument("--geometry", default=None,
                     help="threads,block_size of the headline solve instead of the autotuner's choice")
     ap.add_argument("--only", default=None,

@@ -855,7 +855,7 @@ int dichotomy_plan_ex(double t_m1, double t_0, double t_1, int64_t N, const dich
     // windows of 7-row blocks 6.8 us; N = 600, 10 rows: 8.1 and 6.1), shorter blocks gain nothing.
     // Coupling longer than half a default window, but not half a window of twice the width: with the
     // fixed-point form one pass over overlapping windows is the faster way (tridiag{-1, 2.001, -1},
-    // N = 2^24 + 1: 120 us against 348 us for the general path's two FP64 passes; solved in FP64, where
+    // N = 2^24 + 1: 126 us against 348 us for the general path's two FP64 passes; solved in FP64, where
     // a window's values do not suit fixed point, such windows take about the general path's time).
     // A system with a window for every SM becomes a plan of such windows; a shorter one stays a plan of
     // the general path (what its shards and its plan information are about) whose solves and adjoints
@@ -1583,7 +1583,7 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
   if (!o.NT && o.n_req == 0) {
     // few FP64-form windows are latency-bound.  A batch of nothing else, all of its systems suited to
     // the default windows (fixed point, or at most 16 rows a block), is fastest in these: 154 systems
-    // of 256 to 22682 rows 12.3 us a solve, in 256-thread windows 34.1; 32 of 4096 rows 8.5 and 14.1.
+    // of 256 to 22682 rows 12.8 us a solve, in 256-thread windows 34.1; 32 of 4096 rows 8.5 and 14.1.
     // A handful of ill-conditioned systems beside many MIXED ones (the lowest Poisson modes) takes
     // 256-thread windows of shorter blocks: 300 modes of 2500 rows 17, else 47.
     const int NTd = b->NT[FORM_F64];
@@ -1743,7 +1743,7 @@ int dichotomy_batch_prepare(int64_t nsys, const int64_t* h_N, const int64_t* h_o
     if (q.o_fix || b->adj[(size_t)s].rec.o_fix) b->ntf = 1;
   }
   // threads for windows of at most the default rows: one system of longer blocks would double the CTA of
-  // every window (10000 systems of 256 to 2^20 rows, one of 4033 in 65-row blocks: 8.28 ms, so 5.50).  Its
+  // every window (10000 systems of 256 to 2^20 rows, one of 4033 in 65-row blocks: 8.28 ms, so 5.61).  Its
   // windows are taken as long as their rows fit those threads, in FP64 arithmetic otherwise.
   if (b->ntf)
     b->ntf = fix_threads(b->NT[FORM_F64],

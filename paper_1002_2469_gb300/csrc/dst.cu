@@ -6,8 +6,8 @@
 // Every column has a real FFT of its own: two columns in one complex FFT would each carry rounding errors
 // of the larger one's size, and its Inf and NaN.  (cuFFT itself takes two rows at a time at odd lengths above
 // 256.  A Poisson solve of 2000 x 2319 1363 us, with pairs 1299; 1999 x 2319 922 and 765, 3071 x 3071 1565
-// and 1342.)  The transform's scale sqrt(2 / N) (and the caller's) is folded into the coefficients c1 = scale (s + 1/2), c2 = scale (s - 1/2) of y_k = c1 a_k + c2 a_{N-k},
-// y_{N-k} = c2 a_k + c1 a_{N-k}.
+// and 1342.)  The transform's scale sqrt(2 / N) (and the caller's) is folded into the coefficients
+// c1 = scale (s + 1/2), c2 = scale (s - 1/2) of y_k = c1 a_k + c2 a_{N-k}, y_{N-k} = c2 a_k + c1 a_{N-k}.
 //
 // Each kernel reads and writes its arrays once (the torch expressions they replace made about 15 passes
 // and strided ones among them).  Both move 16 bytes per element; the FP64 pipe (2 operations per clock

@@ -37,14 +37,14 @@
 // coupling over their distance (R per row from the left, B from the right; a lower bound of
 // |T^-1| |F| there, which the FP64 recurrences' errors are relative to), and every level has to
 // reach 2^-lv of the power of two (random right-hand sides do; FX_LVL, fix_table in api.cu).
-// A thread sees its own rows and four on both sides (fix_levels).  Where |F| varies more but smoothly -- from one
-// block of 32 rows to the next by at most `step` binades, 4 to 8 and at most half the decay of the couplings over
-// a block: the spectra and profiles of smooth sources -- every thread takes the largest exponent of its own
-// and its two neighbours' blocks, its levels are held to that (and its unit to kFixSlope binades from the
-// next thread's), and the scans of steps 2 and 4 move signed
-// words between scales.  (What reaches a thread from k + 1 blocks away is then below R^(16 k) <= 2^(-4 k) of
-// its own range: 16/15 into u and again into X, for which K has room or a bit is kept, FX_SPARE.)  Anything else (zero stretches, isolated
-// values, Inf and NaN) is solved in FP64, which resolves a solution's tails relative to themselves.
+// A thread sees its own rows and four on both sides (fix_levels).  Where |F| varies more but smoothly -- from
+// one block of 32 rows to the next by at most `step` binades, 4 to 8 and at most half the decay of the couplings
+// over a block: the spectra and profiles of smooth sources -- every thread takes the largest exponent of its own
+// and its two neighbours' blocks; its levels are held to that, its unit lies at most kFixSlope binades from the
+// next thread's, and the scans of steps 2 and 4 move signed words between scales.  (What reaches a thread from
+// k + 1 blocks away is then below R^(16 k) <= 2^(-4 k) of its own range: 16/15 into u and again into X, for
+// which K has room or a bit is kept, FX_SPARE.)  Anything else (zero stretches, isolated values, Inf and NaN) is
+// solved in FP64, which resolves a solution's tails relative to themselves.
 // (Such a window pays for the copy and the test on top: 33554467 rows with a zero stretch in every window 456 us,
 // in FP64 windows alone 441; 1000003 rows, fewer than two windows an SM, 21.9 and 19.6.)  A window of zeros is its
 // own solution: 33554467 zeros 88 us, solved in FP64 454.
