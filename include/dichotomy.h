@@ -66,7 +66,9 @@ typedef enum {
 
 /* ---------------------------------------------------------------- options */
 typedef enum {
-  DICH_PREC_F64 = 0,    /* every step in FP64 */
+  DICH_PREC_F64 = 0,    /* FP64 accuracy: Toeplitz windows whose values suit it in 64-bit fixed point (a
+                           window's errors, row by row relative to |T^-1| |F|, within those of the FP64
+                           recurrences), every other step in FP64 */
   DICH_PREC_MIXED = 1,  /* local sweeps and spike correction in compensated FP32 (float-float, one
                            power-of-two scale per window); block quantities and the in-window tree
                            in float-float, the general path's block scan in FP64.  Toeplitz plans
